@@ -5,6 +5,19 @@
 // free / unknown / occupied state with the thresholds of Sec. V-A.  A voxel
 // with no kernel mass (never reached, or outside every allocated block) reads
 // as the prior alpha_0 and is unknown.
+//
+// The outputs of 32 consecutive query points are contiguous, so a warp takes
+// 32 points: first a lane per point (hash lookup, the class column into shared
+// memory, the sums), then a lane per output element, which makes every store
+// of the [q, K+1] arrays a full line.  The quotients are formed in pairs of
+// FP32 values (hi + lo, about 2^-46 relative), whose rounding to FP32 is that
+// of the FP64 quotient in all but a 2^-20 share of the cases; FP64 itself runs
+// at 1/64 of the FP32 rate on this chip and bound the kernel before, a lane's
+// stores one sector each: 1.23M points x 20 classes, every output, took
+// 1563 us a call and take 146 us (344 B a point: 62 us at the copy rate); what
+// bounds it now is the lookups' latency and the issue of the pairs' arithmetic.
+// Points whose values leave the pairs' safe range (and states within 1e-9 of a
+// threshold) take the FP64 form.
 #include <algorithm>
 
 #include "sbki_internal.cuh"
@@ -42,57 +55,191 @@ __device__ int32_t lookup_block(const QueryArgs& a, unsigned long long key) {
   return -1;
 }
 
-__global__ void __launch_bounds__(256) query_kernel(QueryArgs a) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.q) return;
+// An unevaluated sum hi + lo of two FP32 values, |lo| at most half an ulp of hi
+// (Dekker's and Knuth's error-free sums and products).
+struct Two {
+  float hi, lo;
+};
+__device__ __forceinline__ Two two_sum(float a, float b) {  // a + b exactly
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Two renorm(float hi, float lo) {
+  const float s = __fadd_rn(hi, lo);
+  return {s, __fsub_rn(lo, __fsub_rn(s, hi))};
+}
+__device__ __forceinline__ Two add(Two a, float b) {
+  const Two s = two_sum(a.hi, b);
+  return renorm(s.hi, __fadd_rn(s.lo, a.lo));
+}
+__device__ __forceinline__ Two mul(Two a, Two b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  const float e = __fmaf_rn(a.hi, b.hi, -p);
+  return renorm(p, __fadd_rn(e, __fmaf_rn(a.hi, b.lo, __fmul_rn(a.lo, b.hi))));
+}
+__device__ __forceinline__ Two recip(Two a) {  // one correction of the rounded reciprocal
+  const float r = __frcp_rn(a.hi);
+  const float e = __fmaf_rn(-r, a.lo, __fmaf_rn(-r, a.hi, 1.0f));
+  return renorm(r, __fmul_rn(r, e));
+}
+
+constexpr int kQWarps = 8;
+// Range in which the pairs keep their accuracy: every alpha zero or at least
+// kMinAlpha, and their sum at most kMaxSum (no factor or residual leaves FP32's
+// normal range; far outside what scans or the default prior produce).
+constexpr float kMinAlpha = 0x1p-30f, kMaxSum = 0x1p40f;
+constexpr int kRowWide = 1 << 8, kRowMode = 1 << 9;  // row flags above the argmax class
+
+// per warp: 32 rows of alpha (odd stride: no bank conflict by lane), then the rows' scalars
+__host__ __device__ constexpr int row_stride(int K1) { return K1 | 1; }
+__host__ __device__ constexpr size_t warp_smem(int K1) { return 32 * (sizeof(float) * (size_t)(row_stride(K1) + 3) + 2 * sizeof(float4)); }
+
+__global__ void __launch_bounds__(32 * kQWarps) query_kernel(QueryArgs a, uint32_t recip_k1) {
+  extern __shared__ __align__(16) unsigned char q_smem[];
   const Geom& g = a.g;
-  const int K1 = g.K1;
-  int v[3];
-  bool inside = true;
+  const int K1 = g.K1, stride = row_stride(K1);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned char* base = q_smem + warp * warp_smem(K1);
+  float4* s_sum = reinterpret_cast<float4*>(base);  // (1/S, S), or S in FP64 in the first two words of a wide row
+  float4* s_rest = s_sum + 32;                      // (S without the largest class, 1/(S + 1))
+  float2* s_mode = reinterpret_cast<float2*>(s_rest + 32);  // 1 / sum (alpha - 1)
+  int* s_flag = reinterpret_cast<int*>(s_mode + 32);
+  float* s_al = reinterpret_cast<float*>(s_flag + 32);
+  const int64_t i0 = ((int64_t)blockIdx.x * kQWarps + warp) * 32, i = i0 + lane;
+  if (i0 >= a.q) return;  // warp-uniform
+  const int rows = (int)min((int64_t)32, a.q - i0);
+  if (i < a.q) {
+    int v[3];
+    bool inside = true;
 #pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    const float s = __fmul_rn(a.xyz[3 * i + ax], g.inv_res);
-    inside = inside && fabsf(s) < (float)(kKeyLimit - 64);
-    v[ax] = inside ? (int)floorf(s) : 0;
-  }
-  int32_t pool = -1;
-  int local = 0;
-  if (inside) {
-    pool = lookup_block(a, pack_block(v[0] >> g.B_shift, v[1] >> g.B_shift, v[2] >> g.B_shift, a.map));
-    const int m = g.B - 1;
-    local = (((v[2] & m) << g.B_shift) + (v[1] & m)) * g.B + (v[0] & m);
-  }
-  const float* inc = pool >= 0 ? a.alpha + (size_t)pool * K1 * g.B3 + local : nullptr;
-  // sums in FP64: 1 - E_k = (S - alpha_k)/S must not cancel when one class dominates
-  double S = 0.0, mass = 0.0;
-  float amax = -1.f, amin = 3.0e38f;
-  int best = 0;
-  for (int k = 0; k < K1; ++k) {
-    const float d = inc ? inc[(size_t)k * g.B3] : 0.f;
-    const float al = a.alpha0 + d;
-    mass += d;
-    S += al;
-    amin = fminf(amin, al);
-    if (al > amax) {
-      amax = al;
-      best = k;
+    for (int ax = 0; ax < 3; ++ax) {
+      const float s = __fmul_rn(a.xyz[3 * i + ax], g.inv_res);
+      inside = inside && fabsf(s) < (float)(kKeyLimit - 64);
+      v[ax] = inside ? (int)floorf(s) : 0;
     }
-  }
-  const bool mode_ok = amin > 1.0f;
-  double po = 0.0;
-  for (int k = 0; k < K1; ++k) {
-    const double al = (double)(a.alpha0 + (inc ? inc[(size_t)k * g.B3] : 0.f));
-    a.probs[i * K1 + k] = (float)(al / S);
-    if (a.var) a.var[i * K1 + k] = (float)(al * (S - al) / (S * S * (S + 1.0)));
-    if (a.mode) a.mode[i * K1 + k] = mode_ok ? (float)((al - 1.0) / (S - (double)K1)) : __int_as_float(0x7fc00000);
-    if (k > 0) po += al / S;
-  }
-  if (a.label) a.label[i] = best;
-  if (a.p_occ) a.p_occ[i] = (float)po;
-  if (a.state) {
+    int32_t pool = -1;
+    int local = 0;
+    if (inside) {
+      pool = lookup_block(a, pack_block(v[0] >> g.B_shift, v[1] >> g.B_shift, v[2] >> g.B_shift, a.map));
+      const int m = g.B - 1;
+      local = (((v[2] & m) << g.B_shift) + (v[1] & m)) * g.B + (v[0] & m);
+    }
+    const float* inc = pool >= 0 ? a.alpha + (size_t)pool * K1 * g.B3 + local : nullptr;
+    float* row = s_al + lane * stride;
+    float amax = -1.f, amin = 3.0e38f;
+    bool any = false, safe = true;  // any: a class with kernel mass
+    int best = 0;
+    constexpr int kAhead = 8;  // class values in flight per lane
+    for (int k0 = 0; k0 < K1; k0 += kAhead) {
+      float d[kAhead];
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j) d[j] = (inc && k0 + j < K1) ? __ldg(inc + (size_t)(k0 + j) * g.B3) : 0.f;
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j)
+        if (k0 + j < K1) {
+          const float al = a.alpha0 + d[j];
+          row[k0 + j] = al;
+          any = any || d[j] > 0.f;
+          safe = safe && d[j] >= 0.f && (al >= kMinAlpha || al == 0.f);
+          amin = fminf(amin, al);
+          if (al > amax) {
+            amax = al;
+            best = k0 + j;
+          }
+        }
+    }
+    // T: every class but the largest, so that S - alpha of the largest class does not cancel
+    Two T = {0.f, 0.f}, M = {0.f, 0.f};
+    for (int k = 0; k < K1; ++k)
+      if (k != best) T = add(T, row[k]);
+    const Two S = add(T, amax);
+    const bool mode_ok = amin > 1.0f;
+    safe = safe && S.hi >= kMinAlpha && S.hi <= kMaxSum;  // false for NaN
+    double wide_s = 0.0, wide_po = 0.0, mass = 0.0;  // the FP64 form
+    auto wide = [&]() {
+      for (int k = 0; k < K1; ++k) {
+        wide_s += row[k];
+        mass += inc ? inc[(size_t)k * g.B3] : 0.f;
+      }
+      for (int k = 1; k < K1; ++k) wide_po += (double)row[k] / wide_s;
+    };
+    float po;
     int st = 1;
-    if (mass > 0.0) st = po < a.free_thresh ? 0 : (po > a.occ_thresh ? 2 : 1);
-    a.state[i] = st;
+    if (safe) {
+      const Two iS = recip(S);
+      Two occ = T;  // classes 1..K
+      if (best != 0) {
+        occ = add(T, -row[0]);
+        occ = add(occ, amax);
+      }
+      const Two p = mul(occ, iS);
+      po = p.hi + p.lo;
+      if (a.state && any) {
+        double pd = (double)p.hi + (double)p.lo;
+        if (fabs(pd - a.free_thresh) < 1e-9 || fabs(pd - a.occ_thresh) < 1e-9) {
+          wide();
+          pd = wide_po;
+        }
+        st = pd < a.free_thresh ? 0 : (pd > a.occ_thresh ? 2 : 1);
+      }
+      if (a.mode && mode_ok) {
+        for (int k = 0; k < K1; ++k) {
+          const Two t = two_sum(row[k], -1.0f);
+          const Two m = add(M, t.hi);
+          M = renorm(m.hi, m.lo + t.lo);
+        }
+        const Two iM = recip(M);
+        s_mode[lane] = make_float2(iM.hi, iM.lo);
+      }
+      const Two iS1 = recip(add(S, 1.0f));
+      s_sum[lane] = make_float4(iS.hi, iS.lo, S.hi, S.lo);
+      s_rest[lane] = make_float4(T.hi, T.lo, iS1.hi, iS1.lo);
+    } else {
+      wide();
+      po = (float)wide_po;
+      if (mass > 0.0) st = wide_po < a.free_thresh ? 0 : (wide_po > a.occ_thresh ? 2 : 1);
+      *reinterpret_cast<double*>(s_sum + lane) = wide_s;
+    }
+    s_flag[lane] = best | (safe ? 0 : kRowWide) | (mode_ok ? kRowMode : 0);
+    if (a.label) a.label[i] = best;
+    if (a.p_occ) a.p_occ[i] = po;
+    if (a.state) a.state[i] = st;
+  }
+  __syncwarp();
+  // a lane per output element of the warp's contiguous rows
+  const int64_t o0 = i0 * K1;
+  const int total = rows * K1;
+  for (int e = lane; e < total; e += 32) {
+    const int r = (int)small_div((uint32_t)e, recip_k1), k = e - r * K1;
+    const int flag = s_flag[r];
+    const float al = s_al[r * stride + k];
+    float mean, var = 0.f, mode = __int_as_float(0x7fc00000);
+    if (flag & kRowWide) {
+      const double S = *reinterpret_cast<const double*>(s_sum + r), al64 = al;
+      mean = (float)(al64 / S);
+      if (a.var) var = (float)(al64 * (S - al64) / (S * S * (S + 1.0)));
+      if (flag & kRowMode) mode = (float)((al64 - 1.0) / (S - (double)K1));
+    } else {
+      const float4 sm = s_sum[r];
+      const Two iS = {sm.x, sm.y}, p = mul({al, 0.f}, iS);
+      mean = p.hi;
+      if (a.var) {
+        const float4 rs = s_rest[r];
+        Two rest = {rs.x, rs.y};  // S - alpha
+        if (k != (flag & 0xff)) {
+          rest = two_sum(sm.z, -al);
+          rest = renorm(rest.hi, rest.lo + sm.w);
+        }
+        var = mul(mul(p, mul(rest, iS)), {rs.z, rs.w}).hi;
+      }
+      if (a.mode && (flag & kRowMode)) {
+        const float2 iM = s_mode[r];
+        mode = mul(two_sum(al, -1.0f), {iM.x, iM.y}).hi;
+      }
+    }
+    a.probs[o0 + e] = mean;
+    if (a.var) a.var[o0 + e] = var;
+    if (a.mode) a.mode[o0 + e] = mode;
   }
 }
 
@@ -119,7 +266,12 @@ cudaError_t launch_query(const MapState& m, const float* xyz, int64_t q, float* 
   a.p_occ = p_occ;
   a.state = state;
   a.map = m.active_map;
-  query_kernel<<<(unsigned)((q + 255) / 256), 256, 0, m.stream>>>(a);
+  // 14 to 35 KB a CTA for 2 to 32 classes: under the 48 KB that need no opt-in
+  static_assert(kQWarps * warp_smem(kMaxClasses) <= 48 * 1024, "read-off shared memory");
+  const int K1 = m.g.K1;
+  const uint32_t recip_k1 = ((1u << 20) + (uint32_t)K1 - 1u) / (uint32_t)K1;
+  const int64_t per = 32 * kQWarps;
+  query_kernel<<<(unsigned)((q + per - 1) / per), 32 * kQWarps, kQWarps * warp_smem(K1), m.stream>>>(a, recip_k1);
   return cudaGetLastError();
 }
 
