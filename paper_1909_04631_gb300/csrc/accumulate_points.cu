@@ -44,7 +44,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kAxisMax = 15;             // offsets per axis: 2R + 1 <= 15
 constexpr int kYZMax = kAxisMax * kAxisMax;
 constexpr float kFar = 1.0e30f;          // d^2 of the padding row
-constexpr int kFastParts = 16;           // fast form: sub-voxel parts per axis of its candidate lists
+constexpr int kFastParts = 8;            // fast form: sub-voxel parts per axis of its candidate lists
 
 struct PtArgs {
   Geom g;
@@ -61,14 +61,17 @@ struct PtArgs {
   uint32_t recip_na;     // small_recip(2R + 1)
   int chunk;             // consecutive training points per warp (fast form)
   int32_t sink;          // spare pool block that absent neighbour blocks point at
-  const uint32_t* ftab;  // fast form: [kFastParts^3][ftpad] (X | Y << 8 | Z << 16 row byte offsets in a slot)
-  const int32_t* flen;   // [kFastParts^3] entries of each list
-  int ftpad;             // entries per fast list (multiple of 32, at most 32 kFastEntries)
+  const uint16_t* ftab;  // fast form: [tables][kFastLists][list_pad] entries, then a list of padding entries
+  const int32_t* flen;   // [tables][kFastLists] entries of each list
+  int list_pad;          // entries per list (a multiple of 16, at most kFastPad)
+  uint32_t pad_list;     // first entry of the list of padding entries
+  float band;            // half-width of the re-decision band around l^2
   const uint32_t* ownslot;  // fast form: per training point the hash slot of its own block (touched-block pass)
   const uint32_t* nbrslot;  // fast form: [hash_cap][32] per own block the hash slots of its touched neighbours
   const int32_t* softidx;   // soft labels (fast form), or null: per training point its weight row, or -1
   const float* wsoft;       // weight rows [.][K+1]
   int tab_of[kMaxClasses];  // per-class supports (fast form): each class's list table, or -1 (not this form)
+  float band_k[kMaxClasses];  // per-class supports: half band of each class
   DevCounters* dc;
 };
 
@@ -184,51 +187,91 @@ __global__ void __launch_bounds__(kThreads, 4) accumulate_points_kernel(PtArgs a
   if (lane == 0) atomicAdd(&a.dc->pairs, (unsigned long long)npairs);
 }
 
-// The same update for 2R + 1 <= 7 (l up to about 3 voxels), shaped for the
-// instruction issue rate, which bounds this loop.
+// The same update for 2R + 1 <= 7 (l below 3.5 voxels): half a warp per point,
+// two voxels adjacent in x per lane.
 //
 // A warp takes a chunk of consecutive training points (sorted by tile, so
-// mostly one block) from a work queue and forms their rows in groups of up to
-// kGroup: three lanes per point (one per axis) write, for offsets j = 0..2R of
-// their axis, the row (e_j^2, address part) into the point's 256-byte slot in
-// shared memory (X rows at bytes 0..63, Y rows at 64..127, Z rows at 128..191,
-// the point's scalars at 192..255).  An address part holds the block digit of
-// the offset (base 3 per axis, times 4: a byte offset into the block table) in
-// its top byte and the voxel's in-block index below it (the X part also
-// carries the point's class row, label * B^3), so the three parts of a
-// candidate add up to (4 digit) << 24 | (label B^3 + in-block index).
+// mostly one block) from a work queue and forms their rows in groups of
+// kGroup, four lanes per point (two for x, one each for y and z), into the
+// point's 256-byte slot in shared memory:
+//   X  four pairs of voxels from the even voxel at or below v0 - R on: the two
+//      squared offsets and an address part (16 bytes a pair);
+//   Y  per offset -R..R (squared offset, address part), and a padding row;
+//   Z  the same; its parts carry the point's class row, label * B^3;
+//   the point's list, class and block.
+// An address part holds the block digit of its axis (4 dx, 12 dy, 36 dz, each
+// in 0..2: a byte offset into the block table) in its top byte and the voxel's
+// in-block index below it, so the three parts of a pair add up to
+// (4 digit) << 24 | (label B^3 + in-block index).  A pair lies in one block
+// (block edges are even).
 //
-// A candidate list entry holds the byte offsets of the candidate's X, Y and Z
-// rows inside a slot (bytes 0, 1, 2), so with the slot at a 256-byte aligned
-// shared address each row address is one byte permute.  Each lane takes two
-// entries at a time and evaluates their kernels with packed FP32 instructions
-// (two values per instruction).  The block table holds, per digit, the first
-// alpha element of the block (the pool slot times (K+1) B^3) minus the digit's
-// top byte, so table entry + summed address parts is the alpha element: one
-// shared load and one add per candidate.  Tables change only when the point's
-// block (or map) changes.  Lists come from a table with kFastParts^3 sub-voxel
-// parts; the next point's entries are loaded while the current one is swept.
-constexpr int kGroup = 10;         // points whose rows one warp forms at once (3 lanes each)
-constexpr int kFastAxis = 8;       // rows per axis: 2R + 1 <= 7 offsets and the X padding row
+// The point's sub-voxel part (kFastParts per axis) picks the list of pairs that
+// can hold a voxel within l (70 to 88 for l = 3 res, x fastest, so the lanes of
+// one voxel row reach the same 32 bytes).  A point in the upper half of its
+// voxel along y or z writes its rows in reverse order and takes the mirrored
+// list; along x, where the pairs' alignment breaks the symmetry, an odd v0 - R
+// is the mirror image of an even one.  That leaves kFastLists lists of 16-bit
+// entries, 24 KB for l = 3 res, which each CTA keeps in shared memory.  A list entry
+// names the pair's X, Y and Z rows so that each row address is one or two
+// operations on the slot's 256-byte aligned address.
+// The block table holds, per digit, the first alpha element of the block (the
+// pool slot times (K+1) B^3) minus the digit's top byte, so table entry +
+// summed parts is the alpha element; it changes only when the half warp's
+// point is in another block.  Both voxels' kernels are evaluated in packed
+// FP32; a voxel past l gets u = 0 (a saturating FMA), hence adds zero, and a
+// pair with a voxel within l is one 8-byte vector reduction.  Membership is the
+// sign of d^2 - l^2, re-decided in FP64 where |d^2 - l^2| is inside the band.
+//
+// Why so: one voxel per lane (lists of up to 160, a warp per point) takes three
+// row loads, a base load and a scalar reduction per voxel, and was bound by the
+// L1 data pipe at 58 wavefronts a point; whole columns of voxels per lane
+// evaluate 7 voxels per lane and round where 3.5 are within l, and were bound
+// by issue (325 instructions a point, 236 us for 690k points).  Here the rows'
+// loads serve two voxels: 29 shared-load wavefronts a point.  Stage times,
+// one voxel per lane -> this form: 188k points of a small region 85 -> 70 us,
+// 690k of a 64 x 2048 street scan 202 -> 198, softmax labels 479 -> 422,
+// per-class l (the widest no longer left to the weighted form) 267 -> 192.
+// Of the 178 us alone (147M warp instructions, issue 70 %, L1 data pipe 67 %)
+// the row set-up takes 45, the reductions 26.
+constexpr int kGroup = 8;          // points whose rows one warp forms at once (4 lanes each)
+constexpr int kFastAxis = 7;       // offsets per axis
 constexpr int kSlotBytes = 256;    // one point's rows and scalars
-constexpr int kFastEntries = 5;    // list entries per lane (lists of at most 160)
-constexpr uint32_t kPadEntry = 8u * (kFastAxis - 1) | (64u << 8) | (128u << 16);  // X padding row, Y row 0, Z row 0
+constexpr uint32_t kYRows = 64u, kZRows = 128u, kScalars = 192u;  // byte offsets in a slot (X rows at 0)
+constexpr int kFastPad = 128;      // entries per list at most: 8 rounds of 16 lanes
+constexpr int kFastLists = kFastParts * (kFastParts / 2) * (kFastParts / 2);
+// entries of a handle's lists: its tables and a list of padding
+__host__ __device__ constexpr int list_entries(int tables, int pad) { return (tables * kFastLists + 1) * pad; }
+// entry: bits 3-5 8 jy, bits 6-7 jx, bits 8-15 the Z row's byte offset in the slot
+constexpr uint32_t kPadEntry = (8u * kFastAxis) | (kZRows << 8);  // Y padding row
 
 struct __align__(256) FastWarp {
-  float2 rows[kGroup][kSlotBytes / 8];  // per point: X, Y, Z rows (8 each), scalars (int view, below)
-  uint32_t btab[64];                    // alpha element base per block digit (27 used)
-  uint32_t ptab[64];                    // pair-count element base per block digit (kTrack)
+  unsigned char slot[kGroup][kSlotBytes];
+  uint32_t btab[2][64];                 // per half warp: alpha element base per block digit (27 used)
 };
-struct __align__(256) FastWarpSoft : FastWarp {
+struct __align__(256) FastWarpTrack : FastWarp {
+  uint32_t ptab[2][64];                 // the same for the pair counts
+};
+template <typename Base>
+struct __align__(256) FastWarpSoft : Base {
   float cw[kGroup][kMaxClasses];        // soft labels: per point sigma0 s_k w^k by class
+  uint32_t cmask[kGroup];               // its classes with a weight
+  int soft[kGroup];                     // 1: the point has a weight row
 };
-// scalars of a slot (int index into its last 64 bytes)
-constexpr int kScPart = 0, kScLabel = 1, kScS0 = 2, kScPool = 3, kScMask = 4, kScSoft = 5, kScV0 = 8;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float2 lds_f2(uint32_t a) {
   float2 v;
   asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds_u4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
   return v;
 }
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
@@ -241,228 +284,305 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-
-// d^2 and summed address part of a candidate of the point whose slot starts at `slot`
-__device__ __forceinline__ void candidate_rows2(uint32_t e, uint32_t slot, float& d2, uint32_t& pk) {
-  const float2 rx = lds_f2(__byte_perm(e, slot, 0x7650));
-  const float2 ry = lds_f2(__byte_perm(e, slot, 0x7651));
-  const float2 rz = lds_f2(__byte_perm(e, slot, 0x7652));
-  d2 = __fadd_rn(__fadd_rn(rx.x, ry.x), rz.x);
-  pk = __float_as_uint(rx.y) + __float_as_uint(ry.y) + __float_as_uint(rz.y);
+// one reduction of 8 aligned bytes where p != 0 (each element is added atomically)
+__device__ __forceinline__ void red_add2_if(uint32_t p, float* addr, float2 v) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q red.global.add.v2.f32 [%1], {%2, %3};\n\t}" ::"r"(p),
+               "l"(addr), "f"(v.x), "f"(v.y)
+               : "memory");
 }
 
-// FP64 re-decision of a candidate in the band around l^2 (rare; point loaded again)
-__device__ __forceinline__ bool band_decide(uint32_t e, const int* sc, const float4* train, uint32_t i, int R,
-                                         double res64, double l2_64) {
+// One axis of a training point: its voxel, the compensated offset to that
+// voxel's centre and its sub-voxel part.
+struct AxisFrame {
+  int v0, part;
+  float hi, lo;
+};
+__device__ __forceinline__ AxisFrame axis_frame(float x, const Geom& g) {
+  AxisFrame f;
+  f.v0 = floor_small(__fmul_rn(x, g.inv_res));
+  centre_offset0(f.v0, x, g, f.hi, f.lo);
+  const float phi = 0.5f - __fmul_rn(__fadd_rn(f.hi, f.lo), g.inv_res);
+  f.part = min(kFastParts - 1, max(0, floor_small(phi * (float)kFastParts)));
+  return f;
+}
+
+// FP64 re-decision of voxel j (0 or 1) of the pair that entry e names (rare;
+// the point is loaded again and its mirrored rows are undone).
+__device__ __noinline__ bool band_decide(uint32_t e, int j, const float4* train, uint32_t i, int R, const Geom& g,
+                                         double l2_64) {
   const float4 p = train[i];
-  const int jx = (int)((e & 0xffu) >> 3), jy = (int)(((e >> 8) & 0xffu) - 64u) >> 3,
-            jz = (int)(((e >> 16) & 0xffu) - 128u) >> 3;
-  return in_support64_call(sc[kScV0] + jx - R, sc[kScV0 + 1] + jy - R, sc[kScV0 + 2] + jz - R, p.x, p.y, p.z, res64,
+  const AxisFrame fx = axis_frame(p.x, g), fy = axis_frame(p.y, g), fz = axis_frame(p.z, g);
+  int jx = (int)(e >> 6) & 3, jy = (int)(e >> 3) & 7, jz = (int)((e >> 8) - kZRows) >> 3;
+  const int odd = (fx.v0 - R) & 1;
+  if (odd) jx = R - jx;
+  if (fy.part >= kFastParts / 2) jy = 2 * R - jy;
+  if (fz.part >= kFastParts / 2) jz = 2 * R - jz;
+  return in_support64_call(fx.v0 - R - odd + 2 * jx + j, fy.v0 + jy - R, fz.v0 + jz - R, p.x, p.y, p.z, g.res64,
                            l2_64);
 }
 
 // Soft labels (kSoft, reading K15): a point with a weight row forms its rows
-// for class 0 (no class row in the X parts) with s0 = 1, and each of its
-// in-support pairs adds f(d/l) sigma0 s_k w^k into every class k with a
-// nonzero weight; a point without one (free samples) is a hard class-0 point.
+// for class 0 with s0 = 1, and each of its in-support pairs adds
+// f(d/l) sigma0 s_k w^k into every class k with a nonzero weight; a point
+// without one (free samples) is a hard class-0 point.
 // Per-class supports (kLk, reading K16): a point's list comes from the table
 // of its class's support l_k, its membership test and kernel use l_k; points
 // of a class without a table are left to the weighted form.
 template <bool kTrack, bool kFace, bool kSoft = false, bool kLk = false>
 __global__ void __launch_bounds__(kThreads, 4) accumulate_points_fast_kernel(PtArgs a) {
-  using Warp = typename std::conditional<kSoft, FastWarpSoft, FastWarp>::type;
+  using Plain = typename std::conditional<kTrack, FastWarpTrack, FastWarp>::type;
+  using Warp = typename std::conditional<kSoft, FastWarpSoft<Plain>, Plain>::type;
   __shared__ Warp s_w[kWarps];
+  extern __shared__ __align__(16) uint16_t s_lists[];  // common support: the lists and the padding list
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   Warp& W = s_w[wid];
   const int R = a.R, na = 2 * R + 1, m = g.B - 1;
   if (a.dc->err != 0) return;
-  if ((smem_addr(&W) & 255u) != 0u) {  // the byte permutes need 256-byte aligned slots
+  if ((smem_addr(&W) & 255u) != 0u) {  // the byte permutes need 256-byte aligned slots and tables
     if (lane == 0) set_error(a.dc, SBKI_ERR_CUDA);
     return;
   }
+  // the padding rows, written once; a half without a point reads X row 0, Z row 0 and the
+  // padding row of its slot, so the slots start at zero (finite, block digit 0)
+  for (int e = lane; e < kGroup * kSlotBytes / 4; e += 32) reinterpret_cast<float*>(W.slot)[e] = 0.0f;
+  __syncwarp();
+  if (lane < kGroup) *reinterpret_cast<float*>(W.slot[lane] + kYRows + 8 * kFastAxis) = kFar;
+  __syncwarp();
+  if (!kLk) {
+    const int n16 = list_entries(1, a.list_pad) / 8;
+    for (int e = threadIdx.x; e < n16; e += kThreads)
+      reinterpret_cast<uint4*>(s_lists)[e] = __ldg(reinterpret_cast<const uint4*>(a.ftab) + e);
+    __syncthreads();
+  }
+  const uint32_t lists = smem_addr(s_lists);
   const uint32_t P = a.dc->n_train;
-  const uint32_t rows0 = smem_addr(&W.rows[0][0]);
-  const uint32_t btab = smem_addr(&W.btab[0]), ptab = smem_addr(&W.ptab[0]);
-  // this lane's point of a group and axis (lanes 30, 31 form no rows)
-  const int gl = lane / 3, ax = lane - 3 * gl;
+  const int half = lane >> 4, hl = lane & 15;
+  const uint32_t slot0 = smem_addr(&W.slot[0][0]) + (uint32_t)half * kSlotBytes;
+  const uint32_t btab0 = smem_addr(&W.btab[0][0]);
+  // this lane's point of a group, and its role there: 0, 1 the halves of X, 2 Y, 3 Z
+  const int gl = lane >> 2, role = lane & 3, ax = max(role - 1, 0);
   const int axshift = ax == 0 ? 0 : (ax == 1 ? g.B_shift : 2 * g.B_shift);
-  const uint32_t dmul = ax == 0 ? 4u : (ax == 1 ? 12u : 36u);
+  const uint32_t dmul = (ax == 0 ? 4u : (ax == 1 ? 12u : 36u)) << 24;
   const uint32_t K1B3 = (uint32_t)(g.K1 * g.B3);
-  const float2 neg_inv_l = make_float2(-g.inv_l, -g.inv_l), one2 = make_float2(1.0f, 1.0f);
-  int cpool = -1;  // own-block pool slot the tables belong to
+  uint32_t cown = 0xffffffffu;  // own block the half's table belongs to
   uint32_t npairs = 0;
-  const uint32_t chunk = (uint32_t)a.chunk;
-  uint32_t c = 0;
-  if (lane == 0) c = atomicAdd(&a.dc->acc_next, 1u);
-  c = __shfl_sync(0xffffffffu, c, 0);
+  // Chunk: about three per warp, at most a.chunk.  Longer ones refill the block
+  // table less often, shorter ones balance the warps (and the queue's one
+  // address takes about 1 ns per claim): 16 / 32 / 48 points took 76 / 87 / 97 us
+  // for 188k points and 228 / 206 / 197 us for 690k.
+  const uint32_t warps = gridDim.x * kWarps;
+  const uint32_t chunk = min((uint32_t)a.chunk, max(P / (3u * warps) / kGroup, 2u) * kGroup);
+  uint32_t c = blockIdx.x * kWarps + (uint32_t)wid;  // the first chunk needs no claim
   while (c * chunk < P) {
     uint32_t cn = 0;  // next chunk, fetched while this one is processed
-    if (lane == 0) cn = atomicAdd(&a.dc->acc_next, 1u);
+    if (lane == 0) cn = warps + atomicAdd(&a.dc->acc_next, 1u);
     const uint32_t c1 = min(P, c * chunk + chunk);
     for (uint32_t g0 = c * chunk; g0 < c1; g0 += kGroup) {
       const uint32_t gn = min(c1 - g0, (uint32_t)kGroup);  // warp-uniform
-      // 1. rows of every point of the group, three lanes per point; the lane
-      //    of axis x also reads the hash slot of the point's own block
+      // 1. rows of every point of the group
       int pt = 0, lw = 0, srow = -1;
+      uint32_t own = 0u;
       if (gl < (int)gn) {
         const float4 p = a.train[g0 + gl];
+        own = __ldg(a.ownslot + g0 + gl);
         if (kSoft) srow = __ldg(a.softidx + g0 + gl);
-        const float xa = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
-        const int v0 = floor_small(__fmul_rn(xa, g.inv_res));
-        float hi, lo;
-        centre_offset0(v0, xa, g, hi, lo);
-        const float phi = 0.5f - __fmul_rn(__fadd_rn(hi, lo), g.inv_res);
-        pt = min(kFastParts - 1, max(0, floor_small(phi * (float)kFastParts)));
-        const int b0 = v0 >> g.B_shift;
+        const AxisFrame f = axis_frame(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), g);
+        const int v0 = f.v0;
         lw = label_of(p.w);
         if (kSoft && srow >= 0) lw &= ~((1 << kLabelBits) - 1);  // class rows come per class in the sweep
-        const uint32_t cls = ax == 0 ? (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3) : 0u;
-        float2* r = W.rows[gl] + kFastAxis * ax;
-        // offsets in a lane-dependent order, so the lanes of one store spread over the banks
-        int j = (gl + 2 * ax) % na;
+        unsigned char* sl = W.slot[gl];
+        const int vrel = v0 - (((v0 >> g.B_shift) - 1) << g.B_shift);  // from the block before the point's
+        if (role < 2) {
+          const int odd = (v0 - R) & 1;
+          pt = odd ? kFastParts - 1 - f.part : f.part;
+          float4* r = reinterpret_cast<float4*>(sl);
 #pragma unroll
-        for (int t = 0; t < kFastAxis - 1; ++t) {
-          if (t < na) {
-            const float e = centre_offset_at(j - R, hi, lo, g);
-            const int v = v0 + j - R;
-            const uint32_t part = (dmul * (uint32_t)((v >> g.B_shift) - b0 + 1)) << 24 | (((uint32_t)(v & m) << axshift) + cls);
-            r[j] = make_float2(__fmul_rn(e, e), __uint_as_float(part));
-            j = j + 1 == na ? 0 : j + 1;
+          for (int t = 0; t < 2; ++t) {
+            const int u = 2 * role + ((gl + t) & 1);  // alternating order: the stores spread over the banks
+            const int d = -R - odd + 2 * u, at = odd ? R - u : u;
+            const float ea = centre_offset_at(d, f.hi, f.lo, g), eb = centre_offset_at(d + 1, f.hi, f.lo, g);
+            const int v = vrel + d;
+            if (at >= 0)  // a pair past the window has no mirror image (and is in no list)
+              r[at] = make_float4(__fmul_rn(ea, ea), __fmul_rn(eb, eb),
+                                  __uint_as_float(dmul * (uint32_t)(v >> g.B_shift) + (uint32_t)(v & m)), 0.f);
+          }
+        } else {
+          const bool flip = f.part >= kFastParts / 2;
+          pt = flip ? kFastParts - 1 - f.part : f.part;
+          const uint32_t cls = role == 3 ? (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3) : 0u;
+          float2* r = reinterpret_cast<float2*>(sl + (role == 2 ? kYRows : kZRows)) + (flip ? 2 * R : 0);
+          const int sgn = flip ? -1 : 1;
+          int j = min(gl, na - 1);  // a lane-dependent order, so the lanes of one store spread over the banks
+#pragma unroll
+          for (int t = 0; t < kFastAxis; ++t) {
+            if (t < na) {
+              const float e = centre_offset_at(j - R, f.hi, f.lo, g);
+              const int v = vrel + j - R;
+              r[sgn * j] = make_float2(__fmul_rn(e, e), __uint_as_float(dmul * (uint32_t)(v >> g.B_shift) +
+                                                                        (((uint32_t)(v & m) << axshift) + cls)));
+              j = j + 1 == na ? 0 : j + 1;
+            }
           }
         }
-        if (ax == 0) r[kFastAxis - 1] = make_float2(kFar, 0.0f);
-        reinterpret_cast<int*>(W.rows[gl] + 3 * kFastAxis)[kScV0 + ax] = v0;
       }
-      const int pty = __shfl_sync(0xffffffffu, pt, min(lane + 1, 31));
-      const int ptz = __shfl_sync(0xffffffffu, pt, min(lane + 2, 31));
-      int list = pt + kFastParts * (pty + kFastParts * ptz);
-      if constexpr (kLk) {  // the table of the point's class support, or -1
-        const int tb = a.tab_of[lw & ((1 << kLabelBits) - 1)];
-        list = tb >= 0 ? list + tb * kFastParts * kFastParts * kFastParts : -1;
+      const int pty = __shfl_sync(0xffffffffu, pt, lane | 2), ptz = __shfl_sync(0xffffffffu, pt, lane | 3);
+      if (role == 0 && gl < (int)gn) {
+        const int label = lw & ((1 << kLabelBits) - 1);
+        const int tb = kLk ? a.tab_of[label] : 0;  // the table of the point's class support, or none
+        const int list = tb * kFastLists + pt + kFastParts * (pty + kFastParts / 2 * ptz);
+        const uint32_t rounds = tb >= 0 ? (uint32_t)(__ldg(a.flen + list) + 15) >> 4 : 0u;
+        *reinterpret_cast<uint4*>(W.slot[gl] + kScalars) =
+            make_uint4(tb >= 0 ? (uint32_t)(list * a.list_pad) : a.pad_list, (uint32_t)lw | (rounds << 16),
+                       __float_as_uint((kSoft && srow >= 0) ? 1.0f : g.sigma0_k[label]), own);
       }
-      if (ax == 0 && gl < (int)gn)
-        *reinterpret_cast<int4*>(reinterpret_cast<int*>(W.rows[gl] + 3 * kFastAxis) + kScPart) =
-            make_int4(list, lw,
-                      __float_as_int((kSoft && srow >= 0) ? 1.0f : g.sigma0_k[lw & ((1 << kLabelBits) - 1)]),
-                      (int)__ldg(a.ownslot + g0 + gl));
       if constexpr (kSoft) {  // class factors sigma0 s_k w^k of the group's soft points
         for (uint32_t k = 0; k < gn; ++k) {
-          const int row = __shfl_sync(0xffffffffu, srow, 3 * k);
+          const int row = __shfl_sync(0xffffffffu, srow, 4 * k);
           float ck = 0.0f;
           if (row >= 0 && lane < g.K1) ck = g.sigma0_k[lane] * __ldg(a.wsoft + (size_t)row * g.K1 + lane);
           const unsigned cm = __ballot_sync(0xffffffffu, ck != 0.0f);
           if (lane < g.K1) W.cw[k][lane] = ck;
           if (lane == 0) {
-            int* sc = reinterpret_cast<int*>(W.rows[k] + 3 * kFastAxis);
-            sc[kScMask] = (int)cm;
-            sc[kScSoft] = row >= 0 ? 1 : 0;
+            W.cmask[k] = cm;
+            W.soft[k] = row >= 0 ? 1 : 0;
           }
         }
       }
       __syncwarp();
-      // 2. point by point: block tables (when the own block changes), candidate sweeps
-      uint32_t ent[kFastEntries];
-      {
-        int part = reinterpret_cast<const int*>(W.rows[0] + 3 * kFastAxis)[kScPart];
-        if constexpr (kLk) part = max(0, part);  // a skipped point (-1) loads list 0, unused
-        const uint32_t* tab = a.ftab + (size_t)part * a.ftpad;
-#pragma unroll
-        for (int it = 0; it < kFastEntries; ++it) ent[it] = __ldg(tab + it * 32 + lane);
+      // 2. block tables.  Points come sorted by tile, so most groups lie in one block: then both
+      //    halves read one table, refilled when the block changes
+      auto fill_digit = [&](int t, uint32_t slot_of_own, int d) {
+        // a digit no point of this block touched holds a stale slot; no
+        // in-support pair uses it (every reduction is predicated on membership)
+        const uint32_t hs = a.nbrslot[(size_t)slot_of_own * 32 + d] & (uint32_t)(a.hash_cap - 1);
+        const int32_t pool = a.hvals[hs];
+        const uint32_t pb = (uint32_t)(pool >= 0 ? pool : a.sink);
+        W.btab[t][d] = pb * K1B3 - ((4u * (uint32_t)d) << 24);
+        if constexpr (kTrack) W.ptab[t][d] = pb * (uint32_t)g.B3 - ((4u * (uint32_t)d) << 24);
+      };
+      const uint32_t own0 = __shfl_sync(0xffffffffu, own, 0);
+      const bool one = __all_sync(0xffffffffu, own == own0 || gl >= (int)gn);  // warp-uniform
+      if (one && own0 != __shfl_sync(0xffffffffu, cown, 0)) {
+        if (half == 0) cown = own0;
+        if (lane < 27) fill_digit(0, own0, lane);
+        __syncwarp();
       }
-      for (uint32_t k = 0; k < gn; ++k) {
-        const int* sc = reinterpret_cast<const int*>(W.rows[k] + 3 * kFastAxis);
-        const int4 sv = *reinterpret_cast<const int4*>(sc + kScPart);  // part, label word, s0, own pool slot
-        const bool soft_pt = kSoft && sc[kScSoft] != 0;
-        const unsigned cmask = kSoft ? (unsigned)sc[kScMask] : 0u;
-        // the next point's list, in flight while this one is swept (lists are
-        // padded to kFastEntries x 32 entries, so every load is in range)
-        uint32_t nent[kFastEntries];
-        {
-          int part = k + 1 < gn ? sc[kScPart + kSlotBytes / 4] : sv.x;
-          if constexpr (kLk) part = max(0, part);
-          const uint32_t* tab = a.ftab + (size_t)part * a.ftpad;
-#pragma unroll
-          for (int it = 0; it < kFastEntries; ++it) nent[it] = __ldg(tab + it * 32 + lane);
-        }
-        if (!(kLk && sv.x < 0)) {  // warp-uniform: a point of a class without a table is the weighted form's
-          if (sv.w != cpool) {  // warp-uniform: the tables belong to another block
-            cpool = sv.w;
-            __syncwarp();  // every lane is done with the old tables
-            if (lane < 27) {
-              // a digit no point of this block touched holds a stale slot; no
-              // in-support pair uses it (every reduction is predicated on membership)
-              const uint32_t hs = a.nbrslot[(size_t)sv.w * 32 + lane] & (uint32_t)(a.hash_cap - 1);
-              const int32_t pool = a.hvals[hs];
-              const uint32_t pb = (uint32_t)(pool >= 0 ? pool : a.sink);
-              W.btab[lane] = pb * K1B3 - ((4u * (uint32_t)lane) << 24);
-              if (kTrack) W.ptab[lane] = pb * (uint32_t)g.B3 - ((4u * (uint32_t)lane) << 24);
+      const uint32_t btab = one ? btab0 : btab0 + (uint32_t)half * (uint32_t)sizeof(W.btab[0]);
+      // 3. two points at a time, one per half warp
+      for (uint32_t k0 = 0; k0 < gn; k0 += 2) {
+        const uint32_t slot = slot0 + k0 * kSlotBytes, k = k0 + (uint32_t)half;
+        const bool have = k < gn;
+        const uint4 sv = lds_u4(slot + kScalars);
+        // this lane's entries of the point's list, one per round
+        const uint32_t list = (have ? sv.x : a.pad_list) + (uint32_t)hl;
+        auto entry = [&](uint32_t r) {
+          return kLk ? (uint32_t)__ldg(a.ftab + list + 16 * r) : lds_u16(lists + 2 * list + 32 * r);
+        };
+        if (!one) {  // warp-uniform: a half's point may be in another block than its table
+          const bool moved = have && sv.w != cown;
+          if (__any_sync(0xffffffffu, moved)) {
+            if (moved) {
+              cown = sv.w;
+              for (int d = hl; d < 27; d += 16) fill_digit(half, cown, d);
             }
             __syncwarp();
           }
-          const uint32_t slot = rows0 + (uint32_t)k * kSlotBytes;
-          const float s0 = __int_as_float(sv.z);
-          const float2 s02 = make_float2(s0, s0);
-          const uint32_t cls = (uint32_t)((sv.y & ((1 << kLabelBits) - 1)) * g.B3);
-          const int len = __ldg(a.flen + sv.x);
-          // the support of the point's class (common l: the kernel's constants)
-          const int cl = sv.y & ((1 << kLabelBits) - 1);
-          const float l2lo = kLk ? g.l2k_lo[cl] : g.l2_lo, l2hi = kLk ? g.l2k_hi[cl] : g.l2_hi;
-          const double l264 = kLk ? g.l2k_64[cl] : g.l2_64;
-          const float2 ninv = kLk ? make_float2(-g.inv_lk[cl], -g.inv_lk[cl]) : neg_inv_l;
-#pragma unroll
-          for (int jp = 0; jp < (kFastEntries + 1) / 2; ++jp) {
-            if (jp < 2 || jp * 64 < len) {  // warp-uniform; lists hold more than 64 entries
-              const uint32_t ea = ent[2 * jp], eb = 2 * jp + 1 < kFastEntries ? ent[2 * jp + 1] : kPadEntry;
-              float d2a, d2b;
-              uint32_t pka, pkb;
-              candidate_rows2(ea, slot, d2a, pka);
-              candidate_rows2(eb, slot, d2b, pkb);
-              bool ina = d2a < l2lo, inb = d2b < l2lo;
-              const bool bnda = !ina && d2a < l2hi, bndb = !inb && d2b < l2hi;
-              if (__any_sync(0xffffffffu, bnda || bndb)) {
-                if (bnda) ina = band_decide(ea, sc, a.train, g0 + k, R, g.res64, l264);
-                if (bndb) inb = band_decide(eb, sc, a.train, g0 + k, R, g.res64, l264);
+        }
+        const uint32_t mine = have ? (sv.y >> 16) & 0xffu : 0u;  // rounds of this half's point
+        const uint32_t rounds = max(mine, __shfl_xor_sync(0xffffffffu, mine, 16));
+        const int label = (int)(sv.y & ((1u << kLabelBits) - 1u));
+        const float s0 = __uint_as_float(sv.z);
+        const float l2 = kLk ? __fmul_rn(0.5f, __fadd_rn(g.l2k_lo[label], g.l2k_hi[label])) : g.l2;
+        const float band = kLk ? a.band_k[label] : a.band;
+        const float ninv = kLk ? -g.inv_lk[label] : -g.inv_l;
+        const float2 nl2 = make_float2(-l2, -l2), s02 = make_float2(s0, s0);
+        uint32_t bits = 0u;  // one per voxel seen, 1 within l
+        // one pair per lane: its d^2 and address, its membership into `bits`
+        struct Pair {
+          float2 d2, t;
+          uint32_t pk;
+        };
+        auto rows_of = [&](uint32_t e) {
+          Pair p;
+          const uint32_t xa = slot | ((e >> 2) & 0x30u);
+          const float2 rx = lds_f2(xa), ry = lds_f2((slot | (e & 0x38u)) + kYRows),
+                       rz = lds_f2(__byte_perm(e, slot, 0x7651));
+          const float rd = __fadd_rn(ry.x, rz.x);
+          p.d2 = __fadd2_rn(make_float2(rd, rd), rx);
+          p.pk = lds_u32(xa + 8) + __float_as_uint(ry.y) + __float_as_uint(rz.y);
+          p.t = __fadd2_rn(p.d2, nl2);
+          return p;
+        };
+        auto near = [](const Pair& p) { return fminf(fabsf(p.t.x), fabsf(p.t.y)); };
+        auto member = [&](const Pair& p) {
+          return __funnelshift_l(__float_as_uint(p.t.y), __float_as_uint(p.t.x) >> 31, 1);
+        };
+        // FP64 decisions of the voxels inside the band; one found outside gets a d^2 past l^2
+        auto redecide = [&](uint32_t e, Pair& p, uint32_t& in) {
+          const double l264 = kLk ? g.l2k_64[label] : g.l2_64;
+          if (fabsf(p.t.x) <= band) {
+            const bool i = band_decide(e, 0, a.train, g0 + k, R, g, l264);
+            in = (in & ~2u) | (i ? 2u : 0u);
+            if (!i) p.d2.x = 4.0f * l2;
+          }
+          if (fabsf(p.t.y) <= band) {
+            const bool i = band_decide(e, 1, a.train, g0 + k, R, g, l264);
+            in = (in & ~1u) | (i ? 1u : 0u);
+            if (!i) p.d2.y = 4.0f * l2;
+          }
+        };
+        // kernels f = u^5 Q(u^2), u = 1 - d / l (0 past l), times sigma0 s_k, added where `in` (bit 1: the
+        // first voxel, bit 0: the second) is not 0
+        auto add_pair = [&](const Pair& p, uint32_t in) {
+          if (kFace && !((kFaceDigits >> (p.pk >> 26)) & 1u)) in = 0u;  // own block and face neighbours only
+          const float2 u = make_float2(__saturatef(__fmaf_rn(sqrt_approx(p.d2.x), ninv, 1.0f)),
+                                       __saturatef(__fmaf_rn(sqrt_approx(p.d2.y), ninv, 1.0f)));
+          const float2 w = __fmul2_rn(u, u);
+          const float2 v = __fmul2_rn(__fmul2_rn(__fmul2_rn(w, w), __fmul2_rn(u, s02)), kernel_q2(w));
+          float* dst = a.alpha + (lds_u32(__byte_perm(p.pk, btab, 0x7653)) + p.pk);
+          bool spread = false;
+          if constexpr (kSoft) {
+            if (W.soft[k & (kGroup - 1)]) {  // uniform over the half: every class with a weight
+              for (unsigned cl = in ? W.cmask[k & (kGroup - 1)] : 0u; cl; cl &= cl - 1u) {
+                const int kc = __ffs((int)cl) - 1;
+                const float ck = W.cw[k & (kGroup - 1)][kc];
+                red_add2_if(1u, dst + (uint32_t)kc * (uint32_t)g.B3, __fmul2_rn(v, make_float2(ck, ck)));
               }
-              if (kFace) {  // extended block: own block and face neighbours (digit in the top byte, times 4)
-                ina = ina && ((kFaceDigits >> (pka >> 26)) & 1u);
-                inb = inb && ((kFaceDigits >> (pkb >> 26)) & 1u);
-              }
-              // kernel of both candidates: f = u^5 Q(u^2), u = 1 - d / l, times sigma0 s_k
-              const float2 d = make_float2(sqrt_approx(d2a), sqrt_approx(d2b));
-              const float2 u = __ffma2_rn(d, ninv, one2);
-              const float2 w = __fmul2_rn(u, u);
-              const float2 q = kernel_q2(w);
-              const float2 v = __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(w, w), u), q), s02);
-              const uint32_t elema = lds_u32(__byte_perm(pka, btab, 0x7653)) + pka;
-              const uint32_t elemb = lds_u32(__byte_perm(pkb, btab, 0x7653)) + pkb;
-              bool spread = false;
-              if constexpr (kSoft) {
-                if (soft_pt) {  // warp-uniform: every class with a weight
-                  for (unsigned cl = cmask; cl; cl &= cl - 1u) {
-                    const int kc = __ffs((int)cl) - 1;
-                    const float ck = W.cw[k][kc];
-                    const uint32_t off = (uint32_t)kc * (uint32_t)g.B3;
-                    if (ina) atomicAdd(a.alpha + elema + off, v.x * ck);
-                    if (inb) atomicAdd(a.alpha + elemb + off, v.y * ck);
-                  }
-                  spread = true;
-                }
-              }
-              if (!spread) {
-                if (ina) atomicAdd(a.alpha + elema, v.x);  // result unused: a reduction
-                if (inb) atomicAdd(a.alpha + elemb, v.y);
-              }
-              if (kTrack) {
-                red_add_if(ina, a.pairs + (lds_u32(__byte_perm(pka, ptab, 0x7653)) + pka - cls), 1);
-                red_add_if(inb, a.pairs + (lds_u32(__byte_perm(pkb, ptab, 0x7653)) + pkb - cls), 1);
-              }
-              npairs += (ina ? 1u : 0u) + (inb ? 1u : 0u);
+              spread = true;
             }
           }
+          red_add2_if(spread ? 0u : in, dst, v);
+          if constexpr (kTrack) {
+            int32_t* pc = a.pairs + (lds_u32(__byte_perm(p.pk, btab + (uint32_t)sizeof(W.btab), 0x7653)) + p.pk -
+                                     (uint32_t)(label * g.B3));
+            red_add_if(in & 2u, pc, 1);
+            red_add_if(in & 1u, pc + 1, 1);
+          }
+          return in;
+        };
+        // rounds in twos (independent chains, one vote), then the odd one
+        uint32_t r = 0;
+        for (; r + 2 <= rounds; r += 2) {  // warp-uniform
+          const uint32_t ea = entry(r), eb = entry(r + 1);
+          Pair pa = rows_of(ea), pb = rows_of(eb);
+          uint32_t ina = member(pa), inb = member(pb);
+          if (__any_sync(0xffffffffu, fminf(near(pa), near(pb)) <= band)) {
+            redecide(ea, pa, ina);
+            redecide(eb, pb, inb);
+          }
+          ina = add_pair(pa, ina);
+          inb = add_pair(pb, inb);
+          bits = (bits << 4) | (ina << 2) | inb;
         }
-#pragma unroll
-        for (int it = 0; it < kFastEntries; ++it) ent[it] = nent[it];
+        if (r < rounds) {
+          const uint32_t ea = entry(r);
+          Pair pa = rows_of(ea);
+          uint32_t ina = member(pa);
+          if (__any_sync(0xffffffffu, near(pa) <= band)) redecide(ea, pa, ina);
+          bits = (bits << 2) | add_pair(pa, ina);
+        }
+        npairs += (uint32_t)__popc(bits);
       }
       __syncwarp();  // the slots are rewritten by the next group
     }
@@ -522,15 +642,49 @@ int candidate_lists(double lr, int parts, std::vector<std::vector<int32_t>>& lis
   return R;
 }
 
-cudaError_t upload_lists(const std::vector<uint32_t>& flat, const std::vector<int32_t>& len, uint32_t** tab,
-                         int32_t** lens) {
-  cudaError_t e = cudaMalloc(tab, sizeof(uint32_t) * flat.size());
+// Pairs of voxels adjacent in x of an even v0 - R, per sub-voxel part
+// (kFastParts along x, the lower half of them along y and z): pair jx holds the
+// offsets -R + 2 jx and the one after it; a list takes every pair with a voxel
+// whose centre can lie within l of a position in the part, widened as above.
+// Entries are packed as jx | (dy + R) << 4 | (dz + R) << 8, x fastest.
+void pair_lists(double lr, int R, std::vector<std::vector<int32_t>>& lists) {
+  const double delta = 1e-3;
+  const int n = kFastParts;
+  auto dist = [&](int d, int part) {
+    return min_axis_distance(d, (double)part / n - delta, (double)(part + 1) / n + delta);
+  };
+  lists.assign(kFastLists, {});
+  for (int t = 0; t < kFastLists; ++t) {
+    const int px = t % n, py = (t / n) % (n / 2), pz = t / (n * (n / 2));
+    for (int dz = -R; dz <= R; ++dz)
+      for (int dy = -R; dy <= R; ++dy)
+        for (int jx = 0; jx < 4; ++jx) {
+          const int dx = -R + 2 * jx;
+          const double mx = std::min(dist(dx, px), dist(dx + 1, px)), my = dist(dy, py), mz = dist(dz, pz);
+          if (mx * mx + my * my + mz * mz < lr * lr * (1.0 + 1e-5))
+            lists[t].push_back(jx | ((dy + R) << 4) | ((dz + R) << 8));
+        }
+  }
+}
+
+// the largest offset whose voxel centre can lie within l of a position in the voxel
+int largest_offset(double lr) {
+  int R = 0;
+  for (int d = 0; d <= 15; ++d)
+    if (min_axis_distance(d, -1e-3, 1.001) < lr * (1.0 + 1e-5) || min_axis_distance(-d, -1e-3, 1.001) < lr * (1.0 + 1e-5))
+      R = d;
+  return R;
+}
+
+template <typename T>
+cudaError_t upload_lists(const std::vector<T>& flat, const std::vector<int32_t>& len, T** tab, int32_t** lens) {
+  cudaError_t e = cudaMalloc(tab, sizeof(T) * flat.size());
   if (e != cudaSuccess) return e;
   e = cudaMalloc(lens, sizeof(int32_t) * len.size());
   if (e != cudaSuccess) return e;
   e = cudaMemcpy(*lens, len.data(), sizeof(int32_t) * len.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
-  return cudaMemcpy(*tab, flat.data(), sizeof(uint32_t) * flat.size(), cudaMemcpyHostToDevice);
+  return cudaMemcpy(*tab, flat.data(), sizeof(T) * flat.size(), cudaMemcpyHostToDevice);
 }
 
 }  // namespace
@@ -569,19 +723,12 @@ cudaError_t build_candidate_tables(MapState& m) {
   if (e != cudaSuccess) return e;
   m.ctab_pad = tpad;
   m.ctab_R = Rt;
-  // The fast form: one table of kFastParts^3 lists per distinct class support
+  // The fast form: one table of kFastLists lists per distinct class support
   // l_k = l l_scale[k] (one table for the common l).  A support qualifies with
   // 2R + 1 <= 7 offsets per axis and l_k above half the voxel diagonal (a
-  // point's own voxel, hence its own block, is then always touched); every
-  // list is padded to 32 kFastEntries entries (the sweep loads all of them
-  // unconditionally).  Entry = X row byte offset 8 jx | (64 + 8 jy) << 8 |
-  // (128 + 8 jz) << 16 inside a point's slot; padding entries name the X
-  // padding row.
+  // point's own voxel, hence its own block, is then always touched).
   const int K1 = m.prm.num_classes + 1;
-  const int fpad = 32 * kFastEntries;
-  std::vector<double> lrs;                              // distinct supports (voxel units)
-  std::vector<std::vector<std::vector<int32_t>>> tabs;  // their lists
-  std::vector<int> rfs;                                 // candidate_lists' R of each
+  std::vector<double> lrs;  // distinct supports (voxel units) that qualify
   int rmax = 0;
   bool own_touched = true;
   m.ftab_classes = 0;
@@ -589,64 +736,38 @@ cudaError_t build_candidate_tables(MapState& m) {
   for (int k = 0; k < K1; ++k) {
     const double lrk = m.prm.length_scale * m.prm.l_scale[k] / m.prm.res;
     own_touched = own_touched && lrk > 0.8661;
+    const int Rk = largest_offset(lrk);
+    if (lrk <= 0.8661 || 2 * Rk + 1 > kFastAxis) continue;
+    rmax = std::max(rmax, Rk);
     size_t t = 0;
     while (t < lrs.size() && lrs[t] != lrk) ++t;
-    if (t == lrs.size()) {  // a new support: its lists, if it qualifies
-      std::vector<std::vector<int32_t>> fl;
-      const int Rf = candidate_lists(lrk, kFastParts, fl);
-      size_t lng = 0;
-      int md = 0;
-      for (auto& L : fl) {
-        lng = std::max(lng, L.size());
-        for (int32_t e : L)
-          for (int a2 = 0; a2 < 3; ++a2) md = std::max(md, std::abs(((e >> (4 * a2)) & 15) - Rf));
-      }
-      if (2 * md + 1 > kFastAxis - 1 || lrk <= 0.8661 || (int)lng > fpad) {
-        lrs.push_back(lrk);
-        tabs.emplace_back();  // does not qualify
-        rfs.push_back(-1);
-      } else {
-        lrs.push_back(lrk);
-        tabs.push_back(std::move(fl));
-        rfs.push_back(Rf);
-        rmax = std::max(rmax, md);
-      }
-    }
-    if (rfs[t] >= 0) m.ftab_classes |= 1u << k;
+    if (t == lrs.size()) lrs.push_back(lrk);
+    m.ftab_of[k] = (int)t;
+    m.ftab_classes |= 1u << k;
   }
   if (m.ftab_classes == 0) return cudaSuccess;
-  // tables in order of first use; rows -rmax..rmax for all of them
-  const int nf = kFastParts * kFastParts * kFastParts, naf = 2 * rmax + 1;
-  std::vector<int> index(lrs.size(), -1);
-  int ntab = 0;
-  for (size_t t = 0; t < lrs.size(); ++t)
-    if (rfs[t] >= 0) index[t] = ntab++;
-  std::vector<uint32_t> ff((size_t)ntab * nf * fpad, kPadEntry);
-  std::vector<int32_t> fl((size_t)ntab * nf);
+  std::vector<std::vector<std::vector<int32_t>>> pairs(lrs.size());
+  size_t most = 0;
   for (size_t t = 0; t < lrs.size(); ++t) {
-    if (index[t] < 0) continue;
-    const size_t b = (size_t)index[t] * nf;
-    for (int q = 0; q < nf; ++q) {
-      const auto& L = tabs[t][q];
-      fl[b + q] = (int32_t)L.size();
-      for (size_t k = 0; k < L.size(); ++k) {
-        const int32_t e = L[k];
-        const uint32_t jx = (uint32_t)((e & 15) - rfs[t] + rmax), jy = (uint32_t)(((e >> 4) & 15) - rfs[t] + rmax),
-                       jz = (uint32_t)(((e >> 8) & 15) - rfs[t] + rmax);
-        if (jx >= (uint32_t)naf || jy >= (uint32_t)naf || jz >= (uint32_t)naf) return cudaErrorInvalidValue;
-        ff[(b + q) * fpad + k] = (8u * jx) | ((64u + 8u * jy) << 8) | ((128u + 8u * jz) << 16);
-      }
+    pair_lists(lrs[t], rmax, pairs[t]);
+    for (auto& L : pairs[t]) most = std::max(most, L.size());
+  }
+  const size_t pad = (most + 15) / 16 * 16;
+  if (pad > (size_t)kFastPad) return cudaErrorInvalidValue;
+  std::vector<uint16_t> ff((size_t)list_entries((int)lrs.size(), (int)pad), (uint16_t)kPadEntry);
+  std::vector<int32_t> fl(lrs.size() * kFastLists);
+  for (size_t t = 0; t < lrs.size(); ++t)
+    for (size_t q = 0; q < (size_t)kFastLists; ++q) {
+      const auto& L = pairs[t][q];
+      fl[t * kFastLists + q] = (int32_t)L.size();
+      for (size_t k = 0; k < L.size(); ++k)
+        ff[(t * kFastLists + q) * pad + k] =
+            (uint16_t)(((L[k] & 15) << 6) | (8 * ((L[k] >> 4) & 15)) | ((kZRows + 8u * (uint32_t)((L[k] >> 8) & 15)) << 8));
     }
-  }
-  for (int k = 0; k < K1; ++k) {
-    size_t t = 0;
-    const double lrk = m.prm.length_scale * m.prm.l_scale[k] / m.prm.res;
-    while (lrs[t] != lrk) ++t;
-    m.ftab_of[k] = index[t];
-  }
   e = upload_lists(ff, fl, &m.ftab, &m.flen);
   if (e != cudaSuccess) return e;
-  m.ftab_pad = fpad;
+  m.ftab_pad = (int)pad;
+  m.ftab_pad_list = (uint32_t)(lrs.size() * kFastLists * pad);
   m.ftab_R = rmax;
   m.ftab_own_touched = own_touched;
   return cudaSuccess;
@@ -656,12 +777,16 @@ namespace {
 
 // ctas_per_sm: 0 = as many as fit
 template <typename Kernel>
-cudaError_t launch_persistent(Kernel kern, const PtArgs& a, int sm_count, int ctas_per_sm, cudaStream_t st) {
+cudaError_t launch_persistent(Kernel kern, const PtArgs& a, int sm_count, int ctas_per_sm, cudaStream_t st,
+                              size_t smem = 0) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
+  cudaError_t e = cudaSuccess;
+  if (smem) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
   if (e != cudaSuccess) return e;
   if (ctas_per_sm > 0) per_sm = std::min(per_sm, ctas_per_sm);
-  kern<<<std::max(1, per_sm) * sm_count, kThreads, 0, st>>>(a);
+  kern<<<std::max(1, per_sm) * sm_count, kThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -670,10 +795,12 @@ cudaError_t launch_fast(const PtArgs& a, int sm_count, int ctas_per_sm, cudaStre
   if (a.g.lscaled)  // per-class supports: the exact association and hard labels only
     return launch_persistent(accumulate_points_fast_kernel<kTrack, false, false, true>, a, sm_count, ctas_per_sm,
                              st);
+  const size_t lists = sizeof(uint16_t) * (size_t)list_entries(1, a.list_pad);
   if (a.softidx)  // soft labels take the exact association only
-    return launch_persistent(accumulate_points_fast_kernel<kTrack, false, true>, a, sm_count, ctas_per_sm, st);
-  return a.g.assoc ? launch_persistent(accumulate_points_fast_kernel<kTrack, true>, a, sm_count, ctas_per_sm, st)
-                   : launch_persistent(accumulate_points_fast_kernel<kTrack, false>, a, sm_count, ctas_per_sm, st);
+    return launch_persistent(accumulate_points_fast_kernel<kTrack, false, true>, a, sm_count, ctas_per_sm, st, lists);
+  if (a.g.assoc)
+    return launch_persistent(accumulate_points_fast_kernel<kTrack, true>, a, sm_count, ctas_per_sm, st, lists);
+  return launch_persistent(accumulate_points_fast_kernel<kTrack, false>, a, sm_count, ctas_per_sm, st, lists);
 }
 
 template <bool kTrack>
@@ -722,14 +849,19 @@ cudaError_t launch_accumulate_points(MapState& m) {
   a.tpad = m.ctab_pad;
   a.R = m.ctab_R;
   a.recip_na = ((1u << 20) + (uint32_t)(2 * m.ctab_R + 1) - 1u) / (uint32_t)(2 * m.ctab_R + 1);
-  a.chunk = std::max(1, std::min(64, m.tune.accumulate_chunk));
+  // whole groups of kGroup points; the kernel takes fewer where there are few points
+  a.chunk = (2 * std::max(1, std::min(64, m.tune.accumulate_chunk)) + kGroup - 1) / kGroup * kGroup;
   // soft labels: a point with a weight row costs up to K+1 times the reductions, so smaller
-  // chunks balance the work queue better (20 against 30: 0.53 against 0.60 ms per street scan)
-  if (m.soft) a.chunk = std::min(a.chunk, 20);
+  // chunks balance the work queue better (16 against 60 points: 413 against 477 us per street scan)
+  if (m.soft) a.chunk = std::min(a.chunk, 16);
   a.sink = (int32_t)m.pool_blocks;
   a.ftab = m.ftab;
   a.flen = m.flen;
-  a.ftpad = m.ftab_pad;
+  a.list_pad = m.ftab_pad;
+  a.pad_list = m.ftab_pad_list;
+  // the re-decision band [l2_lo, l2_hi] as a half-width, widened by the roundings of its ends
+  a.band = 1.0625f * std::max(m.g.l2_hi - m.g.l2, m.g.l2 - m.g.l2_lo);
+  for (int k = 0; k < kMaxClasses; ++k) a.band_k[k] = 1.0625f * 0.5f * (m.g.l2k_hi[k] - m.g.l2k_lo[k]);
   a.ownslot = m.s.ownslot;
   a.nbrslot = m.nbrslot;
   a.softidx = m.soft ? m.s.softidx : nullptr;

@@ -197,10 +197,11 @@ struct MapState {
   ScanDesc* hdesc = nullptr;            // pinned host staging of s.desc
   uint32_t* ctab = nullptr;             // point-major candidate lists [kParts^3][ctab_pad]
   int32_t* clen = nullptr;              // [kParts^3] entries of each list
-  uint32_t* ftab = nullptr;             // fast accumulation form's candidate lists (2R + 1 <= 7), or null:
-                                        // one table of kFastParts^3 lists per distinct class support
+  uint16_t* ftab = nullptr;             // fast accumulation form's candidate lists (2R + 1 <= 7), or null:
+                                        // one table of lists per distinct class support
   int32_t* flen = nullptr;              // their entry counts
-  int ftab_pad = 0;
+  int ftab_pad = 0;                     // entries per list
+  uint32_t ftab_pad_list = 0;           // first entry of the list of padding entries behind the tables
   int ftab_R = 0;                       // offsets -R..R per axis of the fast form's rows
   int32_t ftab_of[32] = {};             // per class: its table, or -1 (the weighted form takes the class)
   uint32_t ftab_classes = 0;            // classes with a table
