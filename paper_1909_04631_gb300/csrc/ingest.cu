@@ -14,15 +14,12 @@
 #include <algorithm>
 #include <climits>
 
-#include "exact_round.cuh"
-#include "sbki_internal.cuh"
+#include "exact_mean.cuh"
 
 namespace sbki {
 namespace {
 
 
-
-__device__ __forceinline__ int floor_i(float v) { return (int)floorf(v); }
 
 // sort key: [scan | rel tile x | rel tile y | rel tile z | local cell (z,y,x) | label]
 __device__ __forceinline__ unsigned long long make_key(float x, float y, float z, int label, const Geom& g,
@@ -50,34 +47,13 @@ __device__ __forceinline__ unsigned long long make_key(float x, float y, float z
   return make_key(x, y, z, label, g, kf, kf.org, 0, dc);
 }
 
-// scan of global point gi: the last s with off[s] <= gi (empty scans are skipped)
-__device__ __forceinline__ int scan_of(const int64_t* off, int ns, int64_t gi) {
-  int lo = 0, hi = ns - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= gi) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 // the map index a training point's segment belongs to
 __device__ __forceinline__ int map_of_segment(unsigned long long key, const KeyFrame& kf, const ScanDesc* desc) {
   return desc[kf.scan_bits ? (int)(key >> kf.total_bits) : 0].map_id;
 }
 
-// number of j >= 1 with fp32(j) * s < r  (the set is a prefix since fp32(j)*s is monotone in j)
-__device__ __forceinline__ uint32_t free_count(float r, float s) {
-  if (!(r > 0.0f)) return 0;
-  float q = __fdiv_rn(r, s);
-  int j = q < 1.6e7f ? (int)q : 16000000;
-  for (int it = 0; it < 4 && j > 0 && !(__fmul_rn((float)j, s) < r); ++it) --j;
-  for (int it = 0; it < 4 && __fmul_rn((float)(j + 1), s) < r; ++it) ++j;
-  return (uint32_t)(j < 0 ? 0 : j);
-}
-
 // a1 for global point i of scan d
-__device__ __forceinline__ void transform_count_one(const ScanDesc& d, int64_t i, const int64_t* off, const Geom& g,
+__device__ __forceinline__ unsigned long long transform_count_one(const ScanDesc& d, int64_t i, const int64_t* off, const Geom& g,
                                                     float4* __restrict__ world, unsigned long long* __restrict__ cnt,
                                                     DevCounters* dc, int tlo[3], int thi[3]) {
   const int64_t li = i - d.off;
@@ -137,22 +113,43 @@ __device__ __forceinline__ void transform_count_one(const ScanDesc& d, int64_t i
   }
   world[i] = w;
   cnt[i] = c;
+  return c;
+}
+
+// the grand total of the per-point counts: hits, free samples, items (capacity check)
+__device__ __forceinline__ void finish_counts(unsigned long long total, int64_t items_cap, DevCounters* dc) {
+  const uint32_t nv = (uint32_t)(total >> 40);
+  const unsigned long long nf = total & kFreeMask;
+  dc->n_valid = nv;
+  dc->n_free = nf;
+  const unsigned long long items = (unsigned long long)nv + nf;
+  dc->n_scan = dc->n_points;
+  if (items > (unsigned long long)items_cap) {
+    set_error(dc, SBKI_ERR_CAPACITY);
+    dc->n_items = dc->n_sort = 0;
+  } else {
+    dc->n_items = dc->n_sort = (uint32_t)items;
+  }
 }
 
 // Steps a1 (and the free-sample counts of a2) for every point of every scan
 // of the update; points are numbered globally, scan after scan.
 __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __restrict__ desc, int ns, Geom g,
                                                                float4* __restrict__ world,
-                                                               unsigned long long* __restrict__ cnt, DevCounters* dc) {
+                                                               unsigned long long* __restrict__ cnt, int64_t items_cap,
+                                                               DevCounters* dc) {
   __shared__ int64_t s_off[kMaxScans + 1];
   __shared__ int s_box[6];
+  __shared__ unsigned long long s_total;
   for (int t = threadIdx.x; t <= ns; t += blockDim.x) s_off[t] = desc[t].off;
   if (threadIdx.x < 6) s_box[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : INT_MIN;
+  if (threadIdx.x == 6) s_total = 0ull;
   __syncthreads();
   const int64_t total = s_off[ns];
   int tlo[3] = {INT_MAX, INT_MAX, INT_MAX}, thi[3] = {INT_MIN, INT_MIN, INT_MIN};
+  unsigned long long sum = 0ull;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tlo, thi);
+    sum += transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tlo, thi);
   // tile bounding box of the kept hits: warp, then CTA, then one global atomic per CTA and bound
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -162,10 +159,22 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
       atomicMax(&s_box[3 + a], hi);
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&s_total, sum);
   __syncthreads();
   if (threadIdx.x < 3 && s_box[threadIdx.x] <= s_box[3 + threadIdx.x]) {
     atomicMin(&dc->tbox[threadIdx.x], s_box[threadIdx.x]);
     atomicMax(&dc->tbox[3 + threadIdx.x], s_box[3 + threadIdx.x]);
+  }
+  if (threadIdx.x == 0) {  // the last CTA to finish (a counter after a fence) has the total
+    atomicAdd(&dc->n_total, s_total);
+    __threadfence();
+    if (atomicAdd(&dc->transform_done, 1u) == gridDim.x - 1) {
+      dc->transform_done = 0u;
+      __threadfence();
+      finish_counts(atomicAdd(&dc->n_total, 0ull), items_cap, dc);
+    }
   }
 }
 
@@ -183,7 +192,7 @@ __global__ void __launch_bounds__(256) emit_kernel(const float4* __restrict__ wo
   __shared__ int64_t s_off[kMaxScans + 1];
   for (int t = threadIdx.x; t <= ns; t += blockDim.x) s_off[t] = desc[t].off;
   __syncthreads();
-  if (dc->err) return;
+  if (dc->err || dc->n_sort == 0u) return;
   const int64_t n = s_off[ns];
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -264,298 +273,15 @@ __global__ void __launch_bounds__(256) emit_kernel(const float4* __restrict__ wo
 // binades, else (and for a mean below the FP32 normal range, or mixed signs) a
 // one-thread signed 512-bit sum, exact for every FP32 input.
 
-struct U128 {
-  unsigned long long lo, hi;
-};
-
-__device__ __forceinline__ float axis_of(const float4& p, int ax) { return ax == 0 ? p.x : (ax == 1 ? p.y : p.z); }
-
-// member i of the sorted order: items already in sorted order (perm null) or gathered through perm
-__device__ __forceinline__ float4 item_at(const float4* __restrict__ items, const uint32_t* __restrict__ perm, uint32_t i) {
-  return perm ? items[perm[i]] : items[i];
-}
-
-// |v| = m 2^e (m < 2^24 integer); returns false for zero
-__device__ __forceinline__ bool decompose(float v, unsigned& m, int& e) {
-  const unsigned b = __float_as_uint(v) & 0x7fffffffu;
-  if (b == 0u) return false;
-  const unsigned E = b >> 23;
-  m = (b & 0x7fffffu) | (E ? 0x800000u : 0u);
-  e = E ? (int)E - 150 : -149;
-  return true;
-}
-
-__device__ __forceinline__ void u128_add(U128& t, unsigned long long lo, unsigned long long hi) {
-  t.lo += lo;
-  t.hi += hi + (t.lo < lo ? 1ull : 0ull);
-}
-
-// t += m 2^sh, 0 <= sh <= 103
-__device__ __forceinline__ void u128_add_shifted(U128& t, unsigned long long m, int sh) {
-  if (sh == 0) u128_add(t, m, 0ull);
-  else if (sh < 64) u128_add(t, m << sh, m >> (64 - sh));
-  else u128_add(t, 0ull, m << (sh - 64));
-}
-
-__device__ __forceinline__ int bitlen64(unsigned long long v) { return v ? 64 - __clzll((long long)v) : 0; }
-
-struct AxisAcc {
-  int emin, emax;  // range of the members' last-mantissa-bit exponents
-  bool neg, pos;   // a member below / above zero
-  __device__ void init() {
-    emin = 1 << 20;
-    emax = -(1 << 20);
-    neg = pos = false;
-  }
-  __device__ void see(float v) {
-    unsigned m;
-    int e;
-    if (decompose(v, m, e)) {
-      emin = min(emin, e);
-      emax = max(emax, e);
-      neg |= v < 0.0f;
-      pos |= v > 0.0f;
-    }
-  }
-  __device__ bool empty() const { return emax < emin; }
-  __device__ bool fits(uint32_t n) const {  // one sign, and T stays below 2^127
-    int lg = 0;
-    while (lg < 32 && (1ull << lg) < n) ++lg;
-    return empty() || (!(neg && pos) && emax - emin + 24 + lg <= 126);
-  }
-  __device__ void add(U128& t, float v) const {
-    unsigned m;
-    int e;
-    if (decompose(v, m, e)) u128_add_shifted(t, m, e - emin);
-  }
-};
-
-// round(T 2^s / n) to FP32; false when the result is below the normal range
-__device__ bool round_mean(U128 T, unsigned long long n, int s, float& out) {
-  const int bt = T.hi ? 64 + bitlen64(T.hi) : bitlen64(T.lo);
-  const int bn = bitlen64(n);
-  const int k = 26 + bn - bt;  // q = floor(T 2^k / n) in [2^24, 2^27)
-  unsigned long long q;
-  bool sticky;
-  if (k >= 0) {
-    const unsigned long long num = T.lo << k;  // bt + k = 26 + bn <= 58 bits
-    q = num / n;
-    sticky = num - q * n != 0ull;
-  } else {
-    const int m = -k;
-    unsigned long long ts, lost;
-    if (m < 64) {
-      ts = (T.lo >> m) | (m ? (T.hi << (64 - m)) : 0ull);
-      lost = T.lo & ((1ull << m) - 1ull);
-    } else {
-      ts = T.hi >> (m - 64);
-      lost = T.lo | (T.hi & ((m - 64 == 0) ? 0ull : ((1ull << (m - 64)) - 1ull)));
-    }
-    q = ts / n;
-    sticky = lost != 0ull || ts - q * n != 0ull;
-  }
-  const int qb = bitlen64(q);
-  if (qb - 1 - k + s < -126) return false;
-  const int sh = qb - 24;
-  unsigned long long mant = q >> sh;
-  const unsigned long long rb = q & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-  if (rb > half || (rb == half && (sticky || (mant & 1ull)))) mant += 1ull;
-  int e = sh - k + s;
-  if (mant == (1ull << 24)) {
-    mant >>= 1;
-    e += 1;
-  }
-  out = ldexpf((float)mant, e);
-  return true;
-}
-
-// One thread: exact mean of axis ax of members [a, b) for any FP32 input.
-// Positive and negative members are summed apart, in 16 32-bit limbs in units
-// of 2^-149 each (512 bits), and the smaller sum is subtracted from the larger.
-__device__ float wide_mean(const float4* __restrict__ items, const uint32_t* __restrict__ perm, uint32_t a,
-                           uint32_t b, int ax) {
-  uint32_t wp[16], wn[16];
-  for (int i = 0; i < 16; ++i) wp[i] = wn[i] = 0u;
-  for (uint32_t i = a; i < b; ++i) {
-    const float v = axis_of(item_at(items, perm, i), ax);
-    unsigned m;
-    int e;
-    if (!decompose(v, m, e)) continue;
-    uint32_t* w = v < 0.0f ? wn : wp;
-    const int sh = e + 149, li = sh >> 5, bi = sh & 31;
-    unsigned long long add = (unsigned long long)m << bi;  // < 2^55
-    for (int j = li; j < 16 && add; ++j) {
-      const unsigned long long t = (unsigned long long)w[j] + (add & 0xffffffffull);
-      w[j] = (uint32_t)t;
-      add = (add >> 32) + (t >> 32);
-    }
-  }
-  bool neg = false;  // the negative members outweigh the positive ones
-  for (int j = 15; j >= 0; --j)
-    if (wn[j] != wp[j]) {
-      neg = wn[j] > wp[j];
-      break;
-    }
-  uint32_t w[16];
-  {
-    const uint32_t* hi = neg ? wn : wp;
-    const uint32_t* lo = neg ? wp : wn;
-    unsigned long long borrow = 0ull;
-    for (int j = 0; j < 16; ++j) {
-      const unsigned long long d = (unsigned long long)hi[j] - lo[j] - borrow;
-      w[j] = (uint32_t)d;
-      borrow = (d >> 63) & 1ull;
-    }
-  }
-  const unsigned long long n = b - a;
-  // quotient of (sum 2^96) / n, limb by limb from the top, in 19 limbs
-  uint32_t q[19];
-  unsigned long long r = 0ull;
-  for (int j = 18; j >= 0; --j) {
-    const unsigned long long cur = (r << 32) | (j >= 3 ? w[j - 3] : 0u);
-    q[j] = (uint32_t)(cur / n);
-    r = cur - (unsigned long long)q[j] * n;
-  }
-  int qb = 0;
-  for (int j = 18; j >= 0 && !qb; --j)
-    if (q[j]) qb = 32 * j + 32 - __clz((int)q[j]);
-  if (qb == 0) return 0.0f;
-  // value = q 2^(-149 - 96); keep 24 bits, fewer for a subnormal result
-  const int lead = qb - 1 - 245;
-  int keep = lead < -126 ? 24 - (-126 - lead) : 24;
-  if (keep < 0) keep = 0;
-  const int drop = qb - keep;
-  auto bit = [&](int i) -> unsigned { return i >= 0 ? (q[i >> 5] >> (i & 31)) & 1u : 0u; };
-  unsigned long long mant = 0ull;
-  for (int i = qb - 1; i >= drop; --i) mant = (mant << 1) | bit(i);
-  bool sticky = r != 0ull;
-  for (int i = 0; i < drop - 1 && !sticky; ++i) sticky = bit(i) != 0u;
-  if (bit(drop - 1) && (sticky || (mant & 1ull))) mant += 1ull;
-  const float f = ldexpf((float)mant, drop - 245);
-  return neg ? -f : f;
-}
-
-__device__ float finish_axis(const AxisAcc& s, bool fits, U128 T, uint32_t n, const float4* items,
-                             const uint32_t* perm, uint32_t a, uint32_t b, int ax) {
-  if (s.empty()) return 0.0f;
-  float f;
-  if (fits && round_mean(T, n, s.emin, f)) return s.neg ? -f : f;
-  return wide_mean(items, perm, a, b, ax);
-}
-
-// Single-pass form for an axis whose first member x0 has |x0| >= 2.5 ds: every
-// member of the cell lies within ds (plus rounding) of x0, so it has x0's sign
-// and its last mantissa bit's exponent is within [e0 - 1, e0 + 1] (e0: x0's);
-// in units of 2^E, E = e0 - 1, every |x| is an integer below 2^26 and a 64-bit
-// sum is exact for fewer than 2^32 members.  Cells near a coordinate plane
-// (|x0| < 2.5 ds) take the two-pass AxisAcc path.
-struct FastAxis {
-  bool on, neg;
-  int E;
-  unsigned long long T;
-  __device__ void init(float x0, float lim) {
-    unsigned m;
-    int e;
-    on = fabsf(x0) >= lim && decompose(x0, m, e);
-    neg = x0 < 0.0f;
-    E = on ? e - 1 : 0;
-    T = 0ull;
-  }
-  __device__ void add(float v) {
-    unsigned m;
-    int e;
-    decompose(v, m, e);  // v != 0: |v| > ds
-    T += (unsigned long long)m << (e - E);
-  }
-  __device__ float finish(uint32_t n) const {
-    U128 t;
-    t.lo = T;
-    t.hi = 0ull;
-    float f = 0.0f;
-    round_mean(t, n, E, f);
-    return neg ? -f : f;
-  }
-};
-
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ U128 warp_sum_u128(U128 t) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, t.lo, o);
-    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, t.hi, o);
-    u128_add(t, lo, hi);
-  }
-  return t;
-}
-
-__device__ __forceinline__ void warp_range(AxisAcc& s) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s.emin = min(s.emin, __shfl_xor_sync(0xffffffffu, s.emin, o));
-    s.emax = max(s.emax, __shfl_xor_sync(0xffffffffu, s.emax, o));
-  }
-  s.neg = __any_sync(0xffffffffu, s.neg);
-  s.pos = __any_sync(0xffffffffu, s.pos);
-}
-
 // Exact mean of a cell the segment pass could not decide (cell s, members
-// [seg_start[s], seg_start[s + 1]) of the sorted items), by a whole warp.  An
-// axis whose first member has |x0| >= 2.5 ds is summed in one pass in 64 bits
-// (FastAxis); any other axis takes its exponent range first, then the 128-bit
-// sum, else wide_mean.
+// [seg_start[s], seg_start[s + 1]) of the sorted items), by a whole warp.
 __device__ void slow_cell(uint32_t s, const unsigned long long* __restrict__ keys, const float4* __restrict__ items,
                           const uint32_t* __restrict__ seg_start, const Geom& g, float4* __restrict__ train,
                           const ScanDesc* __restrict__ desc, const KeyFrame& kf) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t* perm = nullptr;
-  const uint32_t a = seg_start[s], b = seg_start[s + 1], n = b - a;
-  AxisAcc w[3];
-  FastAxis fa[3];
-  U128 t[3];
-  const float4 p0 = item_at(items, perm, a);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    w[c].init();
-    t[c].lo = t[c].hi = 0ull;
-    fa[c].init(axis_of(p0, c), g.fast_lim);
-  }
-  const bool two_pass = !fa[0].on || !fa[1].on || !fa[2].on;  // warp-uniform
-  for (uint32_t i = a + lane; i < b; i += 32) {
-    const float4 p = item_at(items, perm, i);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (fa[c].on) fa[c].add(axis_of(p, c));
-      else w[c].see(axis_of(p, c));
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-    if (fa[c].on) fa[c].T = warp_sum_u64(fa[c].T);
-  bool fit[3] = {false, false, false};
-  if (two_pass) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      warp_range(w[c]);
-      fit[c] = !fa[c].on && w[c].fits(n);
-    }
-    for (uint32_t i = a + lane; i < b; i += 32) {
-      const float4 p = item_at(items, perm, i);
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        if (fit[c]) w[c].add(t[c], axis_of(p, c));
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) t[c] = warp_sum_u128(t[c]);
-  }
-  if (lane == 0) {
-    float out[3];
-    for (int c = 0; c < 3; ++c)
-      out[c] = fa[c].on ? fa[c].finish(n) : finish_axis(w[c], fit[c], t[c], n, items, perm, a, b, c);
+  const uint32_t a = seg_start[s];
+  float out[3] = {0.f, 0.f, 0.f};
+  cell_mean_warp(items, a, seg_start[s + 1], g, out);
+  if ((threadIdx.x & 31u) == 0) {
     const unsigned long long k = keys[a];
     const int label = (int)(k & ((1ull << g.label_bits) - 1));
     train[s] = make_float4(out[0], out[1], out[2], (float)(label + 32 * map_of_segment(k, kf, desc)));
@@ -586,7 +312,6 @@ constexpr int kSegThreads = 256;
 constexpr int kSegPer = 8;
 constexpr int kSegTile = kSegThreads * kSegPer;
 constexpr int kSegWarps = kSegThreads / 32;
-constexpr int kSegShift = 24;      // binades between a tile's |x| bound and its members' smallest last bit
 constexpr uint32_t kSegMaxN = 1u << (63 - 24 - kSegShift);  // |T| < n 2^(24 + kSegShift) < 2^63 below this
 static_assert(kSegTile == kSegTileItems, "segment tile size");
 
@@ -596,7 +321,6 @@ struct SegState {           // sums of a run of members of one cell
   uint32_t flags;           // bit 1 kSegBad: see above; bits 2 + 9a: E + 256 of axis a (the same for every
                             // member of a cell, so runs join by OR)
 };
-constexpr uint32_t kSegBad = 2u;
 
 // Dynamic shared memory: the cells' sums and label words; the first part
 // doubles as the load stage (items, then keys, one pad entry per kSegPer so
@@ -654,12 +378,7 @@ struct SegCarry {   // partial sums of a cell that crosses a tile boundary
 };
 static_assert(sizeof(SegCarry) == kSegCarryBytes, "segment carry layout");
 
-// The sort tile a key names: E per axis packed as in SegState::flags, the
-// scales 2^-E, and kSegBad when a scale is outside the FP32 normal range.
-struct TileUnit {
-  uint32_t meta, bad;
-  float scale[3];
-};
+// The sort tile a key names.
 __device__ __forceinline__ TileUnit tile_unit(unsigned long long key, const Geom& g, const KeyFrame& kf,
                                               const ScanDesc* __restrict__ desc) {
   int o0 = kf.org[0], o1 = kf.org[1], o2 = kf.org[2];
@@ -673,23 +392,8 @@ __device__ __forceinline__ TileUnit tile_unit(unsigned long long key, const Geom
   const int t[3] = {(int)((tile >> (kf.bits[1] + kf.bits[2])) & ((1ull << kf.bits[0]) - 1)) + o0,
                     (int)((tile >> kf.bits[2]) & ((1ull << kf.bits[1]) - 1)) + o1,
                     (int)(tile & ((1ull << kf.bits[2]) - 1)) + o2};
-  TileUnit u;
-  u.meta = 0u;
-  u.bad = 0u;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int mag = t[a] < 0 ? -t[a] : t[a];
-    const float U = __fmul_rn((float)(kTileEdge * mag + kTileEdge + 2), g.ds);
-    const int E = (int)(__float_as_uint(U) >> 23) - 150 - kSegShift;  // |x| < U < 2^(E + 48)
-    u.meta |= (uint32_t)(E + 256) << (2 + 9 * a);
-    const bool ok = E >= -126 && E <= 126;
-    u.scale[a] = ok ? __uint_as_float((uint32_t)(127 - E) << 23) : 0.f;
-    if (!ok) u.bad = kSegBad;
-  }
-  return u;
+  return unit_of_tile(t, g);
 }
-__device__ __forceinline__ int meta_E(uint32_t flags, int a) { return (int)((flags >> (2 + 9 * a)) & 511u) - 256; }
-
 __device__ __forceinline__ void seg_clear(SegState& s) {
   s.T[0] = s.T[1] = s.T[2] = 0ull;
   s.n = 0u;
@@ -708,15 +412,6 @@ __device__ __forceinline__ void seg_add(SegState& s, const TileUnit& u, float x,
     s.T[a] += (unsigned long long)__float2ll_rz(q);
   }
   s.flags |= u.meta | u.bad | (bad ? kSegBad : 0u);
-}
-
-// a := a and b joined (two runs of one cell)
-__device__ __forceinline__ void seg_merge(SegState& a, const SegState& b) {
-  a.T[0] += b.T[0];
-  a.T[1] += b.T[1];
-  a.T[2] += b.T[2];
-  a.n += b.n;
-  a.flags |= b.flags;
 }
 
 // The label word of a training point (label + 32 map) from its cell's key
@@ -763,7 +458,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_count_kernel(const unsigned l
                                                               const DevCounters* dc) {
   __shared__ uint32_t s_w[kSegWarps];
   if (dc->err) return;
-  const int64_t n = min(cap, (int64_t)dc->n_items);
+  const int64_t n = min(cap, (int64_t)dc->n_sort);
   const int64_t nt = (n + kSegTile - 1) / kSegTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) {
@@ -804,7 +499,7 @@ __global__ void __launch_bounds__(kSegThreads, 3) seg_reduce_kernel(
   __shared__ uint32_t s_tile;
   __shared__ int s_cross;      // the tile's last cell goes on in the next tile
   if (dc->err) return;
-  const int64_t n = min(cap, (int64_t)dc->n_items);
+  const int64_t n = min(cap, (int64_t)dc->n_sort);
   const int64_t nt = (n + kSegTile - 1) / kSegTile;
   const uint32_t* counts = work;
   uint32_t* claim = work + ntiles_cap;
@@ -977,7 +672,7 @@ __global__ void __launch_bounds__(256) finish_cells_kernel(const unsigned long l
                                                            const ScanDesc* __restrict__ desc, KeyFrame kf,
                                                            const uint32_t* __restrict__ slow, DevCounters* dc) {
   if (dc->err) return;
-  const int64_t n = min(cap, (int64_t)dc->n_items);
+  const int64_t n = min(cap, (int64_t)dc->n_sort);
   const int64_t nt = (n + kSegTile - 1) / kSegTile;
   const uint32_t ns = dc->n_slow;
   const uint32_t* closing = work + ntiles_cap + 2;
@@ -1101,11 +796,8 @@ inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + thread
 // point count, which the kernels read on the device (dc->n_points, desc[ns].off).
 cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n) {
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(grid_for(total_n, 256), (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm));
-  transform_count_kernel<<<blocks, 256, 0, m.stream>>>(m.s.desc, ns, m.g, m.s.world, m.s.cnt, m.dc);
-  m.launches += 1 + 1;  // transform, prefix sum (which also checks the item count against the capacity)
-  cudaError_t e = exclusive_scan_u64_onepass(m.s.cnt, total_n, m.s.scan_tmp, m.stream, &m.dc->n_points, m.sm_count,
-                                             m.dc, m.s.s_cap);
-  if (e != cudaSuccess) return e;
+  transform_count_kernel<<<blocks, 256, 0, m.stream>>>(m.s.desc, ns, m.g, m.s.world, m.s.cnt, m.s.s_cap, m.dc);
+  m.launches += 1;
   return cudaGetLastError();
 }
 
@@ -1113,6 +805,10 @@ cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf
   const int64_t warps = (total_n + 7) / 8;
   unsigned blocks = (unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm);
   if (blocks == 0) blocks = 1;
+  // the per-point counts become output offsets
+  cudaError_t e = exclusive_scan_u64_onepass(m.s.cnt, total_n, m.s.scan_tmp, m.stream, &m.dc->n_scan, m.sm_count, m.dc);
+  if (e != cudaSuccess) return e;
+  m.launches += 1;
   emit_kernel<<<blocks, 256, 0, m.stream>>>(m.s.world, m.s.cnt, m.s.desc, ns, m.g, kf, m.s.items, m.s.keys, m.s.vals,
                                             hit_src, m.dc);
   m.launches += 1;
@@ -1126,14 +822,14 @@ cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems)
   const int bits = kf.total_bits + kf.scan_bits;
   m.launches += 1 + (bits + 7) / 8 + 3;  // sort, head counts, segment pass, crossing and slow cells
   // the last pass also moves the items into sorted order (s.sitems), so the segment pass reads them in a stream
-  cudaError_t e = radix_sort_pairs(s.keys, s.vals, s.keys2, s.vals2, &m.dc->n_items, nitems, bits, s.hist,
+  cudaError_t e = radix_sort_pairs(s.keys, s.vals, s.keys2, s.vals2, &m.dc->n_sort, nitems, bits, s.hist,
                                    m.sm_count, m.dc, m.stream, s.items, s.sitems);
   if (e != cudaSuccess) return e;
   const int64_t stiles = (nitems + kSegTile - 1) / kSegTile;
   e = cudaMemsetAsync(s.flags + stiles, 0, sizeof(uint32_t) * (stiles + 2), m.stream);
   if (e != cudaSuccess) return e;
-  seg_count_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(stiles, 65535)), kSegThreads, 0, m.stream>>>(
-      s.keys, nitems, s.flags, m.dc);
+  seg_count_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(stiles, 32 * (int64_t)m.sm_count)), kSegThreads, 0,
+                     m.stream>>>(s.keys, nitems, s.flags, m.dc);
   e = cudaFuncSetAttribute(seg_reduce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmemBytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;

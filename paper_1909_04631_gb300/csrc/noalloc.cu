@@ -180,7 +180,7 @@ sbki_status run(const sbki_params* params, const float* points, const int32_t* l
   // count; every other buffer is written before it is read
   DevCounters init;
   memset(&init, 0, sizeof(init));
-  init.n_points = (uint32_t)n;
+  init.n_points = init.max_points = (uint32_t)n;
   for (int a = 0; a < 3; ++a) {
     init.tbox[a] = INT_MAX;
     init.tbox[3 + a] = INT_MIN;

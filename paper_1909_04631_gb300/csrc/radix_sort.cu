@@ -62,9 +62,10 @@ __global__ void __launch_bounds__(kHistThreads) global_hist_kernel(const unsigne
   __shared__ uint32_t h[kMaxPasses][kRadix];
   for (int p = 0; p < passes; ++p) h[p][threadIdx.x] = 0;
   const int64_t stride = (int64_t)gridDim.x * kHistThreads;
-  for (int64_t e = (int64_t)blockIdx.x * kHistThreads + threadIdx.x; e < ntiles * kRadix; e += stride) w.status[0][e] = 0;
-  __syncthreads();
   const int64_t n = dc->err ? 0 : (int64_t)*n_dev;
+  const int64_t used = min(ntiles, (n + kRadixTile - 1) / kRadixTile);  // tiles of this sort
+  for (int64_t e = (int64_t)blockIdx.x * kHistThreads + threadIdx.x; e < used * kRadix; e += stride) w.status[0][e] = 0;
+  __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * kHistThreads + threadIdx.x; i < n; i += stride) {
     const unsigned long long k = keys[i];
     for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(uint32_t)(k >> (8 * p)) & (kRadix - 1)], 1u);

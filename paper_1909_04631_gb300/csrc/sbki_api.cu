@@ -110,7 +110,7 @@ cudaError_t dalloc(T** p, size_t count) {
 }
 
 __global__ void begin_kernel(DevCounters* dc, uint32_t epoch, uint32_t n_points) {
-  dc->n_points = n_points;
+  dc->n_points = dc->max_points = n_points;
   dc->pairs = 0;
   dc->touched_voxels = 0;
   dc->n_free = 0;
@@ -124,6 +124,13 @@ __global__ void begin_kernel(DevCounters* dc, uint32_t epoch, uint32_t n_points)
   dc->n_slow = 0;
   dc->work_next = 0;
   dc->n_soft = 0;
+  dc->n_sort = 0;
+  dc->n_scan = 0;
+  dc->n_total = 0;
+  dc->n_ttiles = 0;
+  dc->n_wide = 0;
+  dc->n_low = 0;
+  dc->n_gather = 0;
   dc->epoch = epoch;
   dc->n_blocks_before = dc->n_blocks;
   for (int a = 0; a < 3; ++a) {
@@ -148,9 +155,19 @@ __global__ void batch_begin_kernel(DevCounters* dc, const ScanDesc* desc, int ns
   dc->n_slow = 0;
   dc->work_next = 0;
   dc->n_soft = 0;
+  dc->n_sort = 0;
+  dc->n_scan = 0;
+  dc->n_total = 0;
+  dc->n_ttiles = 0;
+  dc->n_wide = 0;
+  dc->n_low = 0;
+  dc->n_gather = 0;
   dc->epoch = dc->epoch + 1;
   dc->n_blocks_before = dc->n_blocks;
   dc->n_points = (uint32_t)desc[ns].off;
+  long long most = 0;
+  for (int s = 0; s < ns; ++s) most = max(most, (long long)desc[s].n);
+  dc->max_points = (uint32_t)most;
   for (int a = 0; a < 3; ++a) {
     dc->tbox[a] = INT_MAX;
     dc->tbox[3 + a] = INT_MIN;
@@ -276,6 +293,7 @@ KeyFrame scan_frame(const MapState& m, const double T[16]) {
   const int64_t half = (int64_t)std::ceil((m.prm.max_range + 2.0 * ds) / (kTileEdge * ds)) + 2;
   kf.bits[0] = kf.bits[1] = kf.bits[2] = ceil_log2(2 * half + 1);
   for (int a = 0; a < 3; ++a) {
+    kf.ext[a] = (int32_t)std::min<int64_t>(2 * half + 1, INT_MAX);
     const float o = (float)T[4 * a + 3];
     const float q = o * m.g.inv_ds;
     const int64_t gcell = (int64_t)std::floor(q);
@@ -294,6 +312,7 @@ void fit_frame_to_box(const Geom& g, const int32_t tb[6], const double T[16], Ke
     const int64_t ot = floor_div64((int64_t)std::floor((float)T[4 * a + 3] * g.inv_ds), kTileEdge);
     const int64_t lo = std::min<int64_t>(tb[a], ot) - 1, hi = std::max<int64_t>(tb[3 + a], ot) + 1;
     kf.org[a] = (int32_t)lo;
+    kf.ext[a] = (int32_t)std::min<int64_t>(hi - lo + 1, INT_MAX);
     kf.bits[a] = std::max(1, ceil_log2(hi - lo + 1));
   }
   kf.total_bits = kf.bits[0] + kf.bits[1] + kf.bits[2] + kLocalBits + g.label_bits;
@@ -311,7 +330,9 @@ void fill_desc(ScanDesc& d, const float* pts, const int32_t* labels, int64_t n, 
     d.t[r] = T[4 * r + 3];
     d.o[r] = (float)T[4 * r + 3];
     d.org[r] = kf.org[r];
+    d.ext[r] = kf.ext[r];
   }
+  d.tile0 = 0;
   d.map_id = map;
   d.probs = nullptr;
 }
@@ -456,16 +477,33 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   m.hdesc[1].off = n;
   CK(&m, cudaMemcpyAsync(m.s.desc, m.hdesc, 2 * sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
   CK(&m, launch_transform_count(m, 1, n));
+  // The tile form (soft labels need the sorted items).  Where the frame of
+  // max_range fits a directory, the tiles are marked before the counters come
+  // back, so the read-back also tells how many are occupied.
+  const bool marked = !probs && tile_frame_fits(m, 1, kf);
+  if (marked) CK(&m, launch_tile_mark(m, 1, n, kf));
   st = read_counters(m);
   if (st != SBKI_OK) return st;
   if (m.hc->err != 0) return status_from_device(m);
   *nitems = m.hc->n_items;
   if (*nitems == 0) return SBKI_OK;
+  if (marked && m.hc->n_ttiles <= tile_capacity(m.s.s_cap) && tile_items_fit(m, *nitems)) {
+    CK(&m, launch_tiles(m, 1, n, kf, *nitems));
+    return SBKI_OK;
+  }
   fit_frame_to_box(m.g, m.hc->tbox, T, kf);
-  m.hdesc[0].org[0] = kf.org[0];
-  m.hdesc[0].org[1] = kf.org[1];
-  m.hdesc[0].org[2] = kf.org[2];
+  for (int a = 0; a < 3; ++a) {
+    m.hdesc[0].org[a] = kf.org[a];
+    m.hdesc[0].ext[a] = kf.ext[a];
+  }
   CK(&m, cudaMemcpyAsync(m.s.desc, m.hdesc, sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
+  // a frame fitted to the hits that cannot hold more tiles than there is room for
+  if (!probs && !marked && tile_frame_fits(m, 1, kf) && tile_items_fit(m, *nitems) &&
+      std::min<int64_t>((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2], *nitems) <= tile_capacity(m.s.s_cap)) {
+    CK(&m, launch_tile_mark(m, 1, n, kf));
+    CK(&m, launch_tiles(m, 1, n, kf, *nitems));
+    return SBKI_OK;
+  }
   CK(&m, launch_emit(m, 1, n, kf, probs ? m.s.hit_src : nullptr));
   CK(&m, launch_downsample_n(m, kf, *nitems));
   if (probs) CK(&m, launch_soft_weights(m));
@@ -877,6 +915,7 @@ sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t cou
       dl = m.s.labels + off;
     }
     fill_desc(m.hdesc[i], dp, dl, sc.n, off, sc.pose, scan_frame(m, sc.pose), sc.map_id);
+    m.hdesc[i].tile0 = (uint32_t)((int64_t)i * kf.ext[0] * kf.ext[1] * kf.ext[2]);  // tile form: one frame after another
     off += sc.n;
   }
   m.hdesc[count] = ScanDesc{};
@@ -907,6 +946,11 @@ sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t cou
     batch_begin_kernel<<<1, 1, 0, m.stream>>>(m.dc, m.s.desc, count);
     m.launches += 1;
     cudaError_t ce = launch_transform_count(m, count, m.s.n_cap);
+    // the tile form where the scans' frames fit, then the sorted form for what it leaves (as a rule nothing)
+    if (ce == cudaSuccess && tile_frame_fits(m, count, kf)) {
+      ce = launch_tile_mark(m, count, m.s.n_cap, kf);
+      if (ce == cudaSuccess) ce = launch_tiles(m, count, m.s.n_cap, kf, m.s.s_cap);
+    }
     if (ce == cudaSuccess) ce = launch_emit(m, count, m.s.n_cap, kf);
     if (ce == cudaSuccess) ce = launch_downsample_n(m, kf, m.s.s_cap);
     sbki_status ust = SBKI_OK;

@@ -52,6 +52,15 @@ struct DevCounters {
   uint32_t acc_next;                  // work queue head of the point-major accumulation (reset before it)
   uint32_t n_soft;                    // soft labels: training points with a weight row, this scan
   uint32_t commit_done;               // CTAs of the commit launch finished (the last one commits the count)
+  uint32_t n_sort;                    // items the sorted form downsamples (0 where the tile form takes the update)
+  uint32_t n_scan;                    // points whose sample counts it sums up (likewise)
+  uint32_t transform_done;            // CTAs of the transform finished (the last one adds up the counts)
+  unsigned long long n_total;         // hits << 40 | free samples of this scan
+  uint32_t n_ttiles;                  // tile form: occupied tiles
+  uint32_t n_low;                     // tile form: fractions noted
+  uint32_t n_wide;                    // tile form: training points left to the gathered exact mean
+  uint32_t n_gather;                  // tile form: their members
+  uint32_t max_points;                // points of the update's largest scan
 };
 
 // per-point sample counts of a1/a2: kept hits in bits 40.., free samples below
@@ -100,6 +109,7 @@ struct KeyFrame {
   int bits[3];      // bits of a relative tile index, per axis
   int total_bits;   // bits of a scan-local sort key (the scan index, if any, sits above)
   int scan_bits;    // bits of the scan index in a batched update (0: one scan)
+  int32_t ext[3];   // tiles per axis
 };
 
 // One scan of an update, in device memory (read by the ingest kernels, so a
@@ -113,6 +123,8 @@ struct ScanDesc {
   double r[9], t[3];      // world_from_sensor
   float o[3];             // fp32 sensor origin
   int32_t org[3];         // key-frame origin tile
+  int32_t ext[3];         // tiles of the key frame per axis
+  uint32_t tile0;         // first directory entry of the scan (tile form)
   int32_t map_id;         // target map of the handle
   const float* probs;     // soft labels: [n,K] probability vectors over classes 1..K (device), else null
 };
@@ -324,11 +336,8 @@ constexpr int64_t scan_tmp_bytes_ce(int64_t n) { return 24 * ((n + 2047) / 2048 
 // look-back of tile 1 runs out with SBKI_ERR_TIMEOUT.
 constexpr int64_t kScanSelftestItems = 3 * 2048;
 cudaError_t scan_wait_selftest(unsigned long long* data, void* tmp, DevCounters* dc, cudaStream_t st);
-// items_cap >= 0: data are the per-point sample counts of a1/a2 and the grand
-// total also sets dc->n_valid, n_free and n_items (SBKI_ERR_CAPACITY and no
-// items when they exceed items_cap)
 cudaError_t exclusive_scan_u64_onepass(unsigned long long* data, int64_t n, void* tmp, cudaStream_t st,
-                                       const uint32_t* n_dev, int sm_count, DevCounters* dc, int64_t items_cap = -1);
+                                       const uint32_t* n_dev, int sm_count, DevCounters* dc);
 
 // radix_sort.cu: stable LSD sort of (keys, vals) over bits [0, bits) (at most
 // 8 passes of 8 bits); count read from *n_dev, cap >= count bounds the work
@@ -359,6 +368,15 @@ cudaError_t radix_wait_selftest(unsigned long long* keys, uint32_t* vals, unsign
 cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n);
 cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, uint32_t* hit_src = nullptr);
 cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems);
+// tiles.cu: the downsampling by occupied tiles.  The frame must fit the
+// scratch (tile_frame_fits), the items leave room for the flagged points
+// (tile_items_fit), and the occupied tiles not exceed tile_capacity.
+constexpr int64_t kTileFrameMax = 1 << 22;  // directory entries per scan at most
+int64_t tile_capacity(int64_t sample_capacity);
+bool tile_frame_fits(const MapState& m, int ns, const KeyFrame& kf);
+bool tile_items_fit(const MapState& m, int64_t nitems);
+cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf);
+cudaError_t launch_tiles(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, int64_t nitems);
 cudaError_t launch_train_bbox(MapState& m, const float4* in, int64_t p, int* bbox_dev);
 cudaError_t launch_train_prepare(MapState& m, const float4* in, int64_t p, const KeyFrame& kf);
 

@@ -1,0 +1,100 @@
+"""The downsampling by occupied tiles against the oracle and against the sorted form: the same bits in the same order
+(downsampling tile, cell, label).  Routes: the frame of max_range (marked before the counters are read), the frame
+fitted to the hits (a max_range whose frame is too large), and the sorted form (a scratch without room for the tiles).
+Scans: random clouds on both sides of the coordinate planes, one point, rays along the axes with coordinates too small
+for the sums' unit (points of the gathered mean), hits next to the ground plane (noted fractions, and more of them than
+the list holds), a cell of more than 2^15 members, all 32 classes."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sb():
+    import paper_1909_04631_gb300 as sbm
+    sbm.load()
+    return sbm
+
+
+def _pose(x, y, z, yaw=0.0):
+    T = np.eye(4)
+    T[:2, :2] = [[np.cos(yaw), -np.sin(yaw)], [np.sin(yaw), np.cos(yaw)]]
+    T[:3, 3] = (x, y, z)
+    return T
+
+
+def _scan(kind, rng):
+    if kind == "one":
+        return np.array([[3.2, -1.1, 0.4]], np.float32), _pose(0.1, 0.2, 0.3)
+    if kind == "cloud":
+        return rng.uniform(-9, 9, (3000, 3)).astype(np.float32), _pose(0.7, -0.4, 0.2, 0.3)
+    if kind == "axes":  # directions whose other coordinates are rounding residues, from the origin
+        a = np.repeat(np.arange(4) * (np.pi / 2), 40)
+        r = rng.uniform(1, 20, len(a))
+        p = np.stack([r * np.cos(a), r * np.sin(a), r * 1e-18], 1)
+        q = rng.uniform(-8, 8, (200, 3))
+        q[:, 2] = 3e-41
+        return np.concatenate([p, q]).astype(np.float32), _pose(0, 0, 0)
+    if kind in ("few", "many"):  # hits within the sums' unit of the ground plane: noted one by one, or too many for it
+        p = rng.uniform(-8, 8, (900, 3))
+        k = 40 if kind == "few" else 700
+        p[:k, 2] = rng.uniform(-4e-8, 4e-8, k) - 1.5
+        p[:k, 0] = np.where(np.arange(k) % 7 == 0, -0.25 + rng.uniform(-2e-8, 2e-8, k), p[:k, 0])
+        return p.astype(np.float32), _pose(0.25, 0.1, 1.5)
+    assert kind == "dense"  # members of the cells next to the sensor and along the rays: more than 2^15
+    p = np.array([1.5, 0.7, -0.6]) + 0.03 * rng.random((40000, 3))
+    return p.astype(np.float32), _pose(3.33, -2.2, 1.15)
+
+
+def _order_key(xyz, lab, res):
+    c = np.floor(xyz * np.float32(1 / res)).astype(np.int64)
+    t, l = c >> 3, c & 7
+    return list(zip(t[:, 0], t[:, 1], t[:, 2], l[:, 2], l[:, 1], l[:, 0], lab))
+
+
+@pytest.mark.parametrize("kind", ["one", "cloud", "axes", "few", "many", "dense"])
+@pytest.mark.parametrize("K", [1, 5, 31])
+def test_routes_give_the_oracles_bits(sb, orc, kind, K):
+    rng = np.random.default_rng(len(kind) * 100 + K)
+    pts, T = _scan(kind, rng)
+    lab = rng.integers(1, K + 1, len(pts)).astype(np.int32)
+    sets = []
+    for max_range, cap in ((50.0, 1 << 22), (400.0, 1 << 22), (50.0, None)):
+        prm = dict(res=0.1, length_scale=0.3, sigma0=0.4, alpha0=0.001, free_step=0.3, num_classes=K,
+                   max_range=max_range)
+        ox, ol, st = orc.training_set(orc.params(**prm), pts, lab, T)
+        if cap is None:  # just enough for the items: the directory does not fit
+            cap = st["hits"] + st["free"]
+        with sb.Map(sb.default_params(**prm, pool_blocks=1 << 12, sample_capacity=cap)) as m:
+            gx, gl = m.training_set(pts, lab, T)
+        assert len(gx) == st["train"]
+        sets.append((gx, gl))
+        if kind not in ("axes", "few", "many"):  # a centroid next to a cell's face can round onto it
+            key = _order_key(gx, gl, 0.1)
+            assert sum(a > b for a, b in zip(key, key[1:])) <= len(key) // 1000
+        o, g = np.lexsort((ol, *ox.T)), np.lexsort((gl, *gx.T))
+        np.testing.assert_array_equal(gl[g], ol[o])
+        np.testing.assert_array_equal(gx[g], ox[o])
+    for gx, gl in sets[1:]:
+        np.testing.assert_array_equal(gx, sets[0][0])
+        np.testing.assert_array_equal(gl, sets[0][1])
+
+
+def test_errors_and_recovery(sb):
+    """A label outside the range and a scan beyond the capacity are refused as before, and the map works after."""
+    rng = np.random.default_rng(3)
+    pts = rng.uniform(-9, 9, (500, 3)).astype(np.float32)
+    lab = np.ones(500, np.int32)
+    with sb.Map(sb.default_params(num_classes=3, pool_blocks=1 << 13, sample_capacity=1 << 15)) as m:
+        bad = lab.copy()
+        bad[77] = 4
+        with pytest.raises(sb.SbkiError) as e:
+            m.insert_scan(pts, bad, np.eye(4))
+        assert e.value.status == sb.ERR_LABEL_RANGE
+        far = np.tile(pts * 5, (12, 1))
+        with pytest.raises(sb.SbkiError) as e:
+            m.insert_scan(far, np.ones(len(far), np.int32), np.eye(4))
+        assert e.value.status == sb.ERR_CAPACITY
+        st = m.insert_scan(pts, lab, np.eye(4))
+        assert st["hits"] == 500 and st["train_points"] > 0
