@@ -37,7 +37,8 @@ METRIC = "LiDAR scans/sec (64x2048 street sequence, S-BKI per-scan update)"
 PAIR_CLK_PER_SM = max(14.0 / 128.0, 3.0 / 16.0)
 # sources of the accumulation kernel (a committed DRAM-traffic figure is valid only for these bytes)
 KERNEL_SOURCES = ["paper_1909_04631_gb300/csrc/accumulate_points.cu", "paper_1909_04631_gb300/csrc/kernel_value.cuh",
-                  "paper_1909_04631_gb300/csrc/kernel_poly.cuh", "paper_1909_04631_gb300/csrc/point_common.cuh"]
+                  "paper_1909_04631_gb300/csrc/kernel_poly.cuh", "paper_1909_04631_gb300/csrc/point_common.cuh",
+                  "paper_1909_04631_gb300/csrc/pair_rows.cuh"]
 
 
 def _gen(args):

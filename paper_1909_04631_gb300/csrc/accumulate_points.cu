@@ -34,7 +34,7 @@
 #include <vector>
 
 #include "kernel_value.cuh"
-#include "point_common.cuh"
+#include "pair_rows.cuh"
 
 namespace sbki {
 namespace {
@@ -43,8 +43,6 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kAxisMax = 15;             // offsets per axis: 2R + 1 <= 15
 constexpr int kYZMax = kAxisMax * kAxisMax;
-constexpr float kFar = 1.0e30f;          // d^2 of the padding row
-constexpr int kFastParts = 8;            // fast form: sub-voxel parts per axis of its candidate lists
 
 struct PtArgs {
   Geom g;
@@ -233,17 +231,6 @@ __global__ void __launch_bounds__(kThreads, 4) accumulate_points_kernel(PtArgs a
 // per-class l (the widest no longer left to the weighted form) 267 -> 192.
 // Of the 178 us alone (147M warp instructions, issue 70 %, L1 data pipe 67 %)
 // the row set-up takes 45, the reductions 26.
-constexpr int kGroup = 8;          // points whose rows one warp forms at once (4 lanes each)
-constexpr int kFastAxis = 7;       // offsets per axis
-constexpr int kSlotBytes = 256;    // one point's rows and scalars
-constexpr uint32_t kYRows = 64u, kZRows = 128u, kScalars = 192u;  // byte offsets in a slot (X rows at 0)
-constexpr int kFastPad = 128;      // entries per list at most: 8 rounds of 16 lanes
-constexpr int kFastLists = kFastParts * (kFastParts / 2) * (kFastParts / 2);
-// entries of a handle's lists: its tables and a list of padding
-__host__ __device__ constexpr int list_entries(int tables, int pad) { return (tables * kFastLists + 1) * pad; }
-// entry: bits 3-5 8 jy, bits 6-7 jx, bits 8-15 the Z row's byte offset in the slot
-constexpr uint32_t kPadEntry = (8u * kFastAxis) | (kZRows << 8);  // Y padding row
-
 struct __align__(256) FastWarp {
   unsigned char slot[kGroup][kSlotBytes];
   uint32_t btab[2][64];                 // per half warp: alpha element base per block digit (27 used)
@@ -258,67 +245,11 @@ struct __align__(256) FastWarpSoft : Base {
   int soft[kGroup];                     // 1: the point has a weight row
 };
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ float2 lds_f2(uint32_t a) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint4 lds_u4(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 // one reduction of 8 aligned bytes where p != 0 (each element is added atomically)
 __device__ __forceinline__ void red_add2_if(uint32_t p, float* addr, float2 v) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q red.global.add.v2.f32 [%1], {%2, %3};\n\t}" ::"r"(p),
                "l"(addr), "f"(v.x), "f"(v.y)
                : "memory");
-}
-
-// One axis of a training point: its voxel, the compensated offset to that
-// voxel's centre and its sub-voxel part.
-struct AxisFrame {
-  int v0, part;
-  float hi, lo;
-};
-__device__ __forceinline__ AxisFrame axis_frame(float x, const Geom& g) {
-  AxisFrame f;
-  f.v0 = floor_small(__fmul_rn(x, g.inv_res));
-  centre_offset0(f.v0, x, g, f.hi, f.lo);
-  const float phi = 0.5f - __fmul_rn(__fadd_rn(f.hi, f.lo), g.inv_res);
-  f.part = min(kFastParts - 1, max(0, floor_small(phi * (float)kFastParts)));
-  return f;
-}
-
-// FP64 re-decision of voxel j (0 or 1) of the pair that entry e names (rare;
-// the point is loaded again and its mirrored rows are undone).
-__device__ __noinline__ bool band_decide(uint32_t e, int j, const float4* train, uint32_t i, int R, const Geom& g,
-                                         double l2_64) {
-  const float4 p = train[i];
-  const AxisFrame fx = axis_frame(p.x, g), fy = axis_frame(p.y, g), fz = axis_frame(p.z, g);
-  int jx = (int)(e >> 6) & 3, jy = (int)(e >> 3) & 7, jz = (int)((e >> 8) - kZRows) >> 3;
-  const int odd = (fx.v0 - R) & 1;
-  if (odd) jx = R - jx;
-  if (fy.part >= kFastParts / 2) jy = 2 * R - jy;
-  if (fz.part >= kFastParts / 2) jz = 2 * R - jz;
-  return in_support64_call(fx.v0 - R - odd + 2 * jx + j, fy.v0 + jy - R, fz.v0 + jz - R, p.x, p.y, p.z, g.res64,
-                           l2_64);
 }
 
 // Soft labels (kSoft, reading K15): a point with a weight row forms its rows
@@ -337,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 4) accumulate_points_fast_kernel(PtA
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   Warp& W = s_w[wid];
-  const int R = a.R, na = 2 * R + 1, m = g.B - 1;
+  const int R = a.R;
   if (a.dc->err != 0) return;
   if ((smem_addr(&W) & 255u) != 0u) {  // the byte permutes need 256-byte aligned slots and tables
     if (lane == 0) set_error(a.dc, SBKI_ERR_CUDA);
@@ -362,8 +293,6 @@ __global__ void __launch_bounds__(kThreads, 4) accumulate_points_fast_kernel(PtA
   const uint32_t btab0 = smem_addr(&W.btab[0][0]);
   // this lane's point of a group, and its role there: 0, 1 the halves of X, 2 Y, 3 Z
   const int gl = lane >> 2, role = lane & 3, ax = max(role - 1, 0);
-  const int axshift = ax == 0 ? 0 : (ax == 1 ? g.B_shift : 2 * g.B_shift);
-  const uint32_t dmul = (ax == 0 ? 4u : (ax == 1 ? 12u : 36u)) << 24;
   const uint32_t K1B3 = (uint32_t)(g.K1 * g.B3);
   uint32_t cown = 0xffffffffu;  // own block the half's table belongs to
   uint32_t npairs = 0;
@@ -388,43 +317,10 @@ __global__ void __launch_bounds__(kThreads, 4) accumulate_points_fast_kernel(PtA
         own = __ldg(a.ownslot + g0 + gl);
         if (kSoft) srow = __ldg(a.softidx + g0 + gl);
         const AxisFrame f = axis_frame(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), g);
-        const int v0 = f.v0;
         lw = label_of(p.w);
         if (kSoft && srow >= 0) lw &= ~((1 << kLabelBits) - 1);  // class rows come per class in the sweep
-        unsigned char* sl = W.slot[gl];
-        const int vrel = v0 - (((v0 >> g.B_shift) - 1) << g.B_shift);  // from the block before the point's
-        if (role < 2) {
-          const int odd = (v0 - R) & 1;
-          pt = odd ? kFastParts - 1 - f.part : f.part;
-          float4* r = reinterpret_cast<float4*>(sl);
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const int u = 2 * role + ((gl + t) & 1);  // alternating order: the stores spread over the banks
-            const int d = -R - odd + 2 * u, at = odd ? R - u : u;
-            const float ea = centre_offset_at(d, f.hi, f.lo, g), eb = centre_offset_at(d + 1, f.hi, f.lo, g);
-            const int v = vrel + d;
-            if (at >= 0)  // a pair past the window has no mirror image (and is in no list)
-              r[at] = make_float4(__fmul_rn(ea, ea), __fmul_rn(eb, eb),
-                                  __uint_as_float(dmul * (uint32_t)(v >> g.B_shift) + (uint32_t)(v & m)), 0.f);
-          }
-        } else {
-          const bool flip = f.part >= kFastParts / 2;
-          pt = flip ? kFastParts - 1 - f.part : f.part;
-          const uint32_t cls = role == 3 ? (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3) : 0u;
-          float2* r = reinterpret_cast<float2*>(sl + (role == 2 ? kYRows : kZRows)) + (flip ? 2 * R : 0);
-          const int sgn = flip ? -1 : 1;
-          int j = min(gl, na - 1);  // a lane-dependent order, so the lanes of one store spread over the banks
-#pragma unroll
-          for (int t = 0; t < kFastAxis; ++t) {
-            if (t < na) {
-              const float e = centre_offset_at(j - R, f.hi, f.lo, g);
-              const int v = vrel + j - R;
-              r[sgn * j] = make_float2(__fmul_rn(e, e), __uint_as_float(dmul * (uint32_t)(v >> g.B_shift) +
-                                                                        (((uint32_t)(v & m) << axshift) + cls)));
-              j = j + 1 == na ? 0 : j + 1;
-            }
-          }
-        }
+        const uint32_t cls = (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3);
+        pt = form_rows<true>(W.slot[gl], gl, role, f, cls, R, g);
       }
       const int pty = __shfl_sync(0xffffffffu, pt, lane | 2), ptz = __shfl_sync(0xffffffffu, pt, lane | 3);
       if (role == 0 && gl < (int)gn) {
@@ -724,9 +620,9 @@ cudaError_t build_candidate_tables(MapState& m) {
   m.ctab_pad = tpad;
   m.ctab_R = Rt;
   // The fast form: one table of kFastLists lists per distinct class support
-  // l_k = l l_scale[k] (one table for the common l).  A support qualifies with
-  // 2R + 1 <= 7 offsets per axis and l_k above half the voxel diagonal (a
-  // point's own voxel, hence its own block, is then always touched).
+  // l_k = l l_scale[k] (one table for the common l) of at most 7 offsets per
+  // axis.  The accumulation also needs every l_k above half the voxel diagonal:
+  // a point's own voxel, hence its own block, is then always touched.
   const int K1 = m.prm.num_classes + 1;
   std::vector<double> lrs;  // distinct supports (voxel units) that qualify
   int rmax = 0;
@@ -737,7 +633,7 @@ cudaError_t build_candidate_tables(MapState& m) {
     const double lrk = m.prm.length_scale * m.prm.l_scale[k] / m.prm.res;
     own_touched = own_touched && lrk > 0.8661;
     const int Rk = largest_offset(lrk);
-    if (lrk <= 0.8661 || 2 * Rk + 1 > kFastAxis) continue;
+    if (2 * Rk + 1 > kFastAxis) continue;
     rmax = std::max(rmax, Rk);
     size_t t = 0;
     while (t < lrs.size() && lrs[t] != lrk) ++t;
@@ -829,7 +725,7 @@ cudaError_t launch_fresh_fill(MapState& m) {
 // every point's own block) and addresses alpha and the pair counts with
 // 32-bit element indices
 bool fast_form_ready(const MapState& m) {
-  return m.ftab != nullptr && m.nbrslot != nullptr && (!m.g.lscaled || m.ftab_own_touched) &&
+  return m.ftab != nullptr && m.nbrslot != nullptr && m.ftab_own_touched &&
          (uint64_t)(m.pool_blocks + 1) * (uint64_t)(m.g.K1 * m.g.B3) <= (1ull << 32);
 }
 

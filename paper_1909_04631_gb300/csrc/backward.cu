@@ -27,7 +27,7 @@
 #include <climits>
 
 #include "kernel_value.cuh"
-#include "point_common.cuh"
+#include "pair_rows.cuh"
 
 namespace sbki {
 namespace {
@@ -36,7 +36,6 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kAxisMax = 15;
 constexpr int kYZMax = kAxisMax * kAxisMax;
-constexpr float kFar = 1.0e30f;
 
 // ---------------------------------------------------------------- held-out log-likelihood
 struct LLArgs {
@@ -138,6 +137,11 @@ struct BwdArgs {
   double* acc_class;   // nullable [32]: per class of the point, sum G f
   float* grad_xyz;     // nullable [p][3]: (sigma0 / l) sum G u^4 D (c_v - x)/d
   float xyz_scale;     // sigma0 / l
+  const uint16_t* ftab;  // pair form: lists (as the fast accumulation's)
+  const int32_t* flen;
+  int list_pad, fR;
+  uint32_t pad_list;
+  float band;          // half-width of the re-decision band around l^2
   DevCounters* dc;
 };
 
@@ -256,205 +260,234 @@ __global__ void __launch_bounds__(kThreads, 3) backward_kernel(BwdArgs a) {
   }
 }
 
-// The same pass for 2R + 1 <= 8 with the set-up of the fast accumulation: a
-// warp takes kBwdChunk consecutive training points in groups of up to
-// kBwdGroup; for a group, three lanes per point (one per axis) form the
-// axis's offset rows (e^2, address part, e) for offsets -R..R at once, with
-// the point's sub-voxel part, block and voxel.  Then, point by point, the
-// warp combines the Y and Z rows into YZ rows, refreshes the pool slots of
-// the 27 blocks around the point's block when the block (or map) changed,
-// and sweeps the candidate list in unrolled rounds of 32.  Rows, tests and
-// kernel arithmetic are the ones of backward_kernel, so both give the same
-// pairs and the same FP32 terms.
-constexpr int kBwdGroup = 10;  // points whose rows one warp forms at once (3 lanes each)
-constexpr int kBwdChunk = 20;  // consecutive training points per warp
-constexpr int kBwdAxis = 8;    // rows per axis: 2R + 1 <= 7 offsets and the padding row
+// The same pass in the pair form of the fast accumulation (pair_rows.cuh: half
+// a warp per point, two voxels adjacent in x per lane; the rows hold the offsets
+// themselves here), for supports of at most 7 offsets per axis.  A pair reads
+// its two values of G in one 8-byte load; kernel, slope and the sums are packed
+// FP32.  FP64 runs at 1/64 of the FP32 rate on this chip, so the sums over the
+// points are unevaluated FP32 pairs per lane (error-free sums and products, so
+// as accurate as FP64), joined in FP64 once per warp.
+//
+// Bound by instruction issue, as the accumulation's sweep is.  2.0M points,
+// 223M pairs: one voxel per lane with FP64 sums per point took 1378 us, this
+// form takes 905.  The largest part of the difference are the FP64 sums: two
+// fused multiply-adds per point and lane hold the SM's FP64 units for ~900 us.
+constexpr int kBwdChunk = 16;  // consecutive training points per warp
 
-struct alignas(16) BwdRows {
-  float4 r[3][kBwdAxis];  // per axis: (e^2, address part, e, 0) of offset j - R; r[0][2R + 1] is the padding row
-  int pt[4];              // sub-voxel part per axis, label word
-  int blk[4];             // block per axis
-  int v0[4];              // voxel per axis
+struct __align__(256) BwdWarp {
+  unsigned char slot[kGroup][kSlotBytes];
+  uint32_t btab[2][64];  // per half warp: G element base per block digit (27 used)
 };
 
-struct BwdFastTables {
-  BwdRows pts[kBwdGroup];
-  float4 yz[kBwdAxis * kBwdAxis];  // (e_y^2 + e_z^2, address part, e_y, e_z) of the point being swept
-  const float* blk[27];            // gpool + (pool (K+1) + y_i) B^3, or null
-};
-
-// One candidate of one point: the pair's terms added into sf, sl, sx, sy, sz
-// (the point's coordinates are loaded again only on the FP64 re-decision).
-__device__ __forceinline__ void bwd_candidate(const BwdArgs& a, const BwdFastTables& t, const BwdRows& pr,
-                                              uint32_t ent, int64_t i, float& sf, float& sl, float& sx, float& sy,
-                                              float& sz) {
-  const Geom& g = a.g;
-  const float4 ex = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(pr.r[0]) + 2u * (ent & 0xffu));
-  const float4 eyz = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(t.yz) + 2u * ((ent >> 8) & 0x7ffu));
-  const float d2 = __fadd_rn(ex.x, eyz.x);
-  const int pk = __float_as_int(ex.y) + __float_as_int(eyz.y);
-  bool in = d2 < g.l2_lo;
-  const bool band = !in && d2 < g.l2_hi;
-  if (__any_sync(0xffffffffu, band)) {
-    if (band) {
-      const float4 p = a.xyzl[i];
-      in = in_support64_call(pr.v0[0] + entry_jx(ent) - a.R, pr.v0[1] + entry_jy(ent) - a.R,
-                             pr.v0[2] + entry_jz(ent) - a.R, p.x, p.y, p.z, g.res64, g.l2_64);
-    }
-  }
-  const float* base = t.blk[pk & 0xff];
-  if (in && base != nullptr) {
-    const float G = __ldg(base + (pk >> 8));
-    const float inv_d = rsqrtf(fmaxf(d2, 1e-30f));
-    const float d = d2 * inv_d;
-    const float u = fmaxf(__fmaf_rn(-d, g.inv_l, 1.0f), 0.0f);
-    const float w = u * u;
-    const float u4 = w * w;
-    const float s = G * u4 * kernel_dq(w);  // -G df/dr
-    sf = __fmaf_rn(G * u4 * u, kernel_q(w), sf);
-    sl = __fmaf_rn(s, d, sl);
-    const float c = s * inv_d;
-    sx = __fmaf_rn(c, ex.z, sx);
-    sy = __fmaf_rn(c, eyz.z, sy);
-    sz = __fmaf_rn(c, eyz.w, sz);
-  }
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
-// kNit > 0: lists of exactly kNit x 32 entries, unrolled; 0: any length
-template <int kNit>
-__global__ void __launch_bounds__(kThreads, 3) backward_fast_kernel(BwdArgs a) {
-  __shared__ BwdFastTables s_tab[kWarps];
+// Running sums of two quantities as unevaluated pairs hi + lo.
+struct PairSum {
+  float2 hi, lo;
+  __device__ __forceinline__ void add(float2 v, float s) {  // += s v, exactly up to the pair's 2^-48
+    const float2 s2 = make_float2(s, s), p = __fmul2_rn(v, s2);
+    const float2 e = __ffma2_rn(v, s2, make_float2(-p.x, -p.y));
+    const float2 t = __fadd2_rn(hi, p);
+    const float2 b = __fadd2_rn(t, make_float2(-hi.x, -hi.y));
+    const float2 d = __fadd2_rn(hi, __fadd2_rn(b, make_float2(-t.x, -t.y)));  // hi - (t - b)
+    const float2 f = __fadd2_rn(p, make_float2(-b.x, -b.y));
+    lo = __fadd2_rn(lo, __fadd2_rn(e, __fadd2_rn(d, f)));
+    hi = t;
+  }
+  __device__ __forceinline__ double total() const {
+    return ((double)hi.x + (double)hi.y) + ((double)lo.x + (double)lo.y);
+  }
+};
+
+template <bool kClass>
+__global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) {
+  __shared__ BwdWarp s_w[kWarps];
+  __shared__ double s_cls[kClass ? kWarps : 1][32];  // per warp: sum G f by class
+  extern __shared__ __align__(16) uint16_t s_lists[];
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int R = a.R, na = 2 * R + 1, m = g.B - 1;
-  BwdFastTables& t = s_tab[wid];
-  __shared__ double s_cls[kWarps][32];  // per warp: sum G f by class (only with acc_class)
+  BwdWarp& W = s_w[wid];
+  const int R = a.fR;
   if (a.dc->err != 0) return;
-  s_cls[wid][lane] = 0.0;
-  // this lane's point of a group and axis (lanes 30, 31 form no rows)
-  const int gl = lane / 3, ax = lane - 3 * (lane / 3);
-  const int axshift = ax == 0 ? 0 : (ax == 1 ? g.B_shift : 2 * g.B_shift);
-  const int dmul = ax == 0 ? 1 : (ax == 1 ? 3 : 9);
-  int cb[3] = {INT_MIN, INT_MIN, INT_MIN}, cmap = -1;  // block and map the cached slots belong to
-  int32_t pool = -1;                                   // lanes 0..26: slot of block digit `lane`
-  double acc_f = 0.0, acc_l = 0.0;
+  if ((smem_addr(&W) & 255u) != 0u) {  // the byte permutes need 256-byte aligned slots and tables
+    if (lane == 0) set_error(a.dc, SBKI_ERR_CUDA);
+    return;
+  }
+  // a half without a point reads X row 0, Z row 0 and the padding row of its slot
+  for (int e = lane; e < kGroup * kSlotBytes / 4; e += 32) reinterpret_cast<float*>(W.slot)[e] = 0.0f;
+  __syncwarp();
+  if (lane < kGroup) *reinterpret_cast<float*>(W.slot[lane] + kYRows + 8 * kFastAxis) = kFarOffset;
+  if (kClass) s_cls[wid][lane] = 0.0;
+  const int n16 = list_entries(1, a.list_pad) / 8;
+  for (int e = threadIdx.x; e < n16; e += kThreads)
+    reinterpret_cast<uint4*>(s_lists)[e] = __ldg(reinterpret_cast<const uint4*>(a.ftab) + e);
+  __syncthreads();
+  const uint32_t lists = smem_addr(s_lists);
+  const int half = lane >> 4, hl = lane & 15;
+  const uint32_t slot0 = smem_addr(&W.slot[0][0]) + (uint32_t)half * kSlotBytes;
+  const uint32_t btab = smem_addr(&W.btab[half][0]);
+  const int gl = lane >> 2, role = lane & 3, ax = max(role - 1, 0);
+  const uint32_t K1B3 = (uint32_t)(g.K1 * g.B3);
+  unsigned long long cblk = kEmpty;  // block the half's table belongs to
+  uint32_t present = 0u;             // its digits that are in the map
+  PairSum acc_f, acc_l;              // sum s G f, sum s G u^4 D d, by column
+  acc_f.hi = acc_f.lo = acc_l.hi = acc_l.lo = make_float2(0.f, 0.f);
+  const int64_t gw = (int64_t)blockIdx.x * kWarps + wid, nw = (int64_t)gridDim.x * kWarps;
   for (int64_t c = gw; c * kBwdChunk < a.p; c += nw) {
     const int64_t c1 = min(a.p, c * kBwdChunk + kBwdChunk);
-    for (int64_t g0 = c * kBwdChunk; g0 < c1; g0 += kBwdGroup) {
-      const int gn = (int)min(c1 - g0, (int64_t)kBwdGroup);  // warp-uniform
-      // 1. rows of every point of the group, three lanes per point
+    for (int64_t g0 = c * kBwdChunk; g0 < c1; g0 += kGroup) {
+      const int gn = (int)min(c1 - g0, (int64_t)kGroup);  // warp-uniform
+      // rows of every point of the group, four lanes per point
+      int pt = 0, lw = 0, b0 = 0;
       if (gl < gn) {
         const float4 p = a.xyzl[g0 + gl];
-        const float xa = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
-        const int v0 = floor_small(__fmul_rn(xa, g.inv_res));
-        float hi, lo;
-        centre_offset0(v0, xa, g, hi, lo);
-        const float phi = 0.5f - __fmul_rn(__fadd_rn(hi, lo), g.inv_res);
-        const int b0 = v0 >> g.B_shift;
-        BwdRows& pr = t.pts[gl];
-#pragma unroll
-        for (int j = 0; j < kBwdAxis; ++j) {
-          if (j < na) {
-            const float e = centre_offset_at(j - R, hi, lo, g);
-            const int v = v0 + j - R;
-            pr.r[ax][j] = make_float4(__fmul_rn(e, e),
-                                      __int_as_float(dmul * ((v >> g.B_shift) - (b0 - 1)) | ((v & m) << (axshift + 8))),
-                                      e, 0.f);
-          }
-        }
-        if (ax == 0) pr.r[0][na] = make_float4(kFar, __int_as_float(0), 0.f, 0.f);
-        pr.pt[ax] = min(kParts - 1, max(0, floor_small(phi * (float)kParts)));
-        pr.blk[ax] = b0;
-        pr.v0[ax] = v0;
-        if (ax == 0) pr.pt[3] = label_of(p.w);
+        const AxisFrame f = axis_frame(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), g);
+        lw = label_of(p.w);
+        pt = form_rows<false>(W.slot[gl], gl, role, f, (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3), R, g);
+        b0 = f.v0 >> g.B_shift;
+      }
+      const int pty = __shfl_sync(0xffffffffu, pt, lane | 2), ptz = __shfl_sync(0xffffffffu, pt, lane | 3);
+      const int by = __shfl_sync(0xffffffffu, b0, lane | 2), bz = __shfl_sync(0xffffffffu, b0, lane | 3);
+      if (role == 0 && gl < gn) {
+        const int list = pt + kFastParts * (pty + kFastParts / 2 * ptz);
+        const int label = lw & ((1 << kLabelBits) - 1), map = lw >> kLabelBits;
+        const bool known = label < g.K1 && map < kMaxMaps;  // others have no G
+        const unsigned long long key = known ? pack_block(b0, by, bz, map) : kEmpty;
+        uint32_t* sc = reinterpret_cast<uint32_t*>(W.slot[gl] + kScalars);
+        sc[0] = known ? (uint32_t)(list * a.list_pad) : a.pad_list;
+        sc[1] = (uint32_t)(label & 31) | (known ? (uint32_t)(__ldg(a.flen + list) + 15) >> 4 : 0u) << 16;
+        sc[2] = (uint32_t)key;
+        sc[3] = (uint32_t)(key >> 32);
       }
       __syncwarp();
-      // 2. point by point: YZ rows, block slots, candidate sweeps, the point's terms
-      for (int k = 0; k < gn; ++k) {
-        const BwdRows& pr = t.pts[k];
-        const int4 ip = *reinterpret_cast<const int4*>(pr.pt);
-        const int4 ib = *reinterpret_cast<const int4*>(pr.blk);
-        const int part = ip.x + kParts * (ip.y + kParts * ip.z);
-        const int label = ip.w & ((1 << kLabelBits) - 1), map = ip.w >> kLabelBits;
-        for (int q0 = 0; q0 < na * na; q0 += 32) {
-          const int q = min(q0 + lane, na * na - 1);
-          const int jy = (int)small_div((uint32_t)q, a.recip_na), jz = q - jy * na;
-          const float4 ry = pr.r[1][jy], rz = pr.r[2][jz];
-          if (q0 + lane < na * na)
-            t.yz[q] = make_float4(__fadd_rn(ry.x, rz.x), __int_as_float(__float_as_int(ry.y) + __float_as_int(rz.y)),
-                                  ry.z, rz.z);
-        }
-        if (ib.x != cb[0] || ib.y != cb[1] || ib.z != cb[2] || map != cmap) {  // warp-uniform
-          cb[0] = ib.x;
-          cb[1] = ib.y;
-          cb[2] = ib.z;
-          cmap = map;
-          pool = -1;
-          if (lane < 27 && map < kMaxMaps)
-            pool = find_pool_slot(a.hkeys, a.hvals, a.hash_cap,
-                                  pack_block(ib.x - 1 + lane % 3, ib.y - 1 + (lane / 3) % 3, ib.z - 1 + lane / 9, map));
-        }
-        if (lane < 27)
-          t.blk[lane] = (pool >= 0 && label < g.K1) ? a.gpool + ((size_t)pool * g.K1 + label) * g.B3 : nullptr;
-        __syncwarp();
-        const uint32_t* tab = a.ctab + part * a.tpad;
-        const int len = __ldg(a.clen + part);
-        const int64_t i = g0 + k;
-        float sf = 0.f, sl = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
-        if (kNit > 0) {
-          uint32_t ent[kNit > 0 ? kNit : 1];
-#pragma unroll
-          for (int it = 0; it < kNit; ++it) ent[it] = it * 32 < len ? __ldg(tab + it * 32 + lane) : 0u;
-#pragma unroll
-          for (int it = 0; it < kNit; ++it)
-            if (it * 32 < len) bwd_candidate(a, t, pr, ent[it], i, sf, sl, sx, sy, sz);  // warp-uniform
-        } else {
-          for (int q = lane; q - lane < len; q += 32) bwd_candidate(a, t, pr, __ldg(tab + q), i, sf, sl, sx, sy, sz);
-        }
-        const float s = label < g.K1 ? g.scale_k[label] : 0.f;  // the class's kernel scale
-        acc_f += (double)s * (double)sf;
-        acc_l += (double)s * (double)sl;
-        if (a.acc_class) add_class_sum(s_cls[wid], label, sf, lane);
-        if (a.grad_xyz) {
-          for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_down_sync(0xffffffffu, sx, o);
-            sy += __shfl_down_sync(0xffffffffu, sy, o);
-            sz += __shfl_down_sync(0xffffffffu, sz, o);
+      // two points at a time, one per half warp
+      for (int k0 = 0; k0 < gn; k0 += 2) {
+        const uint32_t slot = slot0 + (uint32_t)k0 * kSlotBytes;
+        const int k = k0 + half;
+        const bool have = k < gn;
+        const uint4 sv = lds_u4(slot + kScalars);
+        const unsigned long long key = (unsigned long long)sv.w << 32 | sv.z;
+        const bool moved = have && key != kEmpty && key != cblk;
+        if (__any_sync(0xffffffffu, moved)) {  // a half's table belongs to another block
+          uint32_t in = 0u;
+          if (moved) {
+            cblk = key;
+            int bx, byy, bzz;
+            unpack_block(key, bx, byy, bzz);
+            const int map = map_of_block(key);
+            for (int d = hl; d < 27; d += 16) {
+              const int32_t pool = find_pool_slot(a.hkeys, a.hvals, a.hash_cap,
+                                                  pack_block(bx - 1 + d % 3, byy - 1 + (d / 3) % 3, bzz - 1 + d / 9, map));
+              in |= pool >= 0 ? 1u << d : 0u;
+              W.btab[half][d] = (pool >= 0 ? (uint32_t)pool : 0u) * K1B3 - ((4u * (uint32_t)d) << 24);
+            }
           }
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) in |= __shfl_xor_sync(0xffffffffu, in, o);
+          if (moved) present = in;
+          __syncwarp();
+        }
+        const uint32_t mine = have ? (sv.y >> 16) & 0xffu : 0u;  // rounds of this half's point
+        const uint32_t rounds = max(mine, __shfl_xor_sync(0xffffffffu, mine, 16));
+        const uint32_t list = lists + 2u * ((mine ? sv.x : a.pad_list) + (uint32_t)hl);
+        const float2 nl2 = make_float2(-g.l2, -g.l2);
+        float2 sf = make_float2(0.f, 0.f), sl = sf;  // sum G f, sum G u^4 D d of this lane's two columns
+        float2 gx = sf, gy = sf, gz = sf;
+        for (uint32_t r = 0; r < rounds; ++r) {  // warp-uniform
+          const uint32_t e = lds_u16(list + 32u * r);
+          const uint32_t xa = slot | ((e >> 2) & 0x30u);
+          const float2 ex = lds_f2(xa), ry = lds_f2((slot | (e & 0x38u)) + kYRows),
+                       rz = lds_f2(__byte_perm(e, slot, 0x7651));
+          const float rd = __fadd_rn(__fmul_rn(ry.x, ry.x), __fmul_rn(rz.x, rz.x));
+          const float2 d2 = __fadd2_rn(make_float2(rd, rd), __fmul2_rn(ex, ex));
+          const uint32_t pk = lds_u32(xa + 8) + __float_as_uint(ry.y) + __float_as_uint(rz.y);
+          const float2 t = __fadd2_rn(d2, nl2);
+          bool ina = t.x < 0.f, inb = t.y < 0.f;
+          if (__any_sync(0xffffffffu, fminf(fabsf(t.x), fabsf(t.y)) <= a.band)) {
+            if (fabsf(t.x) <= a.band) ina = band_decide(e, 0, a.xyzl, (uint32_t)(g0 + k), R, g, g.l2_64);
+            if (fabsf(t.y) <= a.band) inb = band_decide(e, 1, a.xyzl, (uint32_t)(g0 + k), R, g, g.l2_64);
+          }
+          const uint32_t dig = pk >> 26;
+          float2 G = make_float2(0.f, 0.f);
+          if ((ina || inb) && ((present >> dig) & 1u))
+            G = __ldg(reinterpret_cast<const float2*>(a.gpool + (lds_u32(__byte_perm(pk, btab, 0x7653)) + pk)));
+          if (!ina) G.x = 0.f;
+          if (!inb) G.y = 0.f;
+          const float2 id = make_float2(rsqrt_approx(fmaxf(d2.x, 1e-30f)), rsqrt_approx(fmaxf(d2.y, 1e-30f)));
+          const float2 d = __fmul2_rn(d2, id);
+          const float2 u = make_float2(__saturatef(__fmaf_rn(-d.x, g.inv_l, 1.0f)),
+                                       __saturatef(__fmaf_rn(-d.y, g.inv_l, 1.0f)));
+          const float2 w = __fmul2_rn(u, u);
+          const float2 Gu4 = __fmul2_rn(G, __fmul2_rn(w, w));
+          const float2 s = __fmul2_rn(Gu4, kernel_dq2(w));  // -G df/dr
+          sf = __ffma2_rn(__fmul2_rn(Gu4, u), kernel_q2(w), sf);
+          sl = __ffma2_rn(s, d, sl);
+          const float2 c2 = __fmul2_rn(s, id);
+          // e = c_v - x and dr/dx = -e/(l d), so dk/dx = sigma0 u^4 D e / (l d)
+          gx = __ffma2_rn(c2, ex, gx);
+          gy = __ffma2_rn(c2, make_float2(ry.x, ry.x), gy);
+          gz = __ffma2_rn(c2, make_float2(rz.x, rz.x), gz);
+        }
+        const int label = (int)(sv.y & 31u);
+        const float s = mine ? g.scale_k[label] : 0.f;  // the class's kernel scale
+        acc_f.add(sf, s);
+        acc_l.add(sl, s);
+        if (kClass) {
+          float v = mine ? sf.x + sf.y : 0.f;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          const float v1 = __shfl_sync(0xffffffffu, v, 16);
+          const int l1 = __shfl_sync(0xffffffffu, label, 16);
           if (lane == 0) {
-            a.grad_xyz[3 * i] = sx * (s * a.xyz_scale);
-            a.grad_xyz[3 * i + 1] = sy * (s * a.xyz_scale);
-            a.grad_xyz[3 * i + 2] = sz * (s * a.xyz_scale);
+            s_cls[wid][label] += (double)v;
+            s_cls[wid][l1] += (double)v1;
           }
         }
-        __syncwarp();  // the YZ rows and block pointers are rewritten for the next point
+        if (a.grad_xyz) {
+          // joined over the half's lanes; lanes 0, 1, 2 of a half write x, y, z
+          float sx = gx.x + gx.y, sy = gy.x + gy.y, sz = gz.x + gz.y;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) {
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+            sz += __shfl_xor_sync(0xffffffffu, sz, o);
+          }
+          if (have && hl < 3) a.grad_xyz[3 * (g0 + k) + hl] = (hl == 0 ? sx : (hl == 1 ? sy : sz)) * (s * a.xyz_scale);
+        }
       }
+      __syncwarp();  // the slots are rewritten by the next group
     }
   }
+  double af = acc_f.total(), al = acc_l.total();
   for (int o = 16; o > 0; o >>= 1) {
-    acc_f += __shfl_down_sync(0xffffffffu, acc_f, o);
-    acc_l += __shfl_down_sync(0xffffffffu, acc_l, o);
+    af += __shfl_down_sync(0xffffffffu, af, o);
+    al += __shfl_down_sync(0xffffffffu, al, o);
   }
   if (lane == 0) {
-    atomicAdd(&a.acc[0], acc_f);
-    atomicAdd(&a.acc[1], acc_l);
+    atomicAdd(&a.acc[0], af);
+    atomicAdd(&a.acc[1], al);
   }
-  if (a.acc_class) {
+  if (kClass) {
     __syncwarp();
     if (s_cls[wid][lane] != 0.0) atomicAdd(&a.acc_class[lane], s_cls[wid][lane]);
   }
 }
 
-template <int kNit>
-cudaError_t launch_backward_fast(const BwdArgs& a, int sm_count, cudaStream_t st) {
+template <bool kClass>
+cudaError_t launch_backward_pairs(const BwdArgs& a, int sm_count, cudaStream_t st) {
+  const size_t smem = sizeof(uint16_t) * (size_t)list_entries(1, a.list_pad);
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_fast_kernel<kNit>, kThreads, 0);
+  cudaError_t e = cudaFuncSetAttribute(backward_pairs_kernel<kClass>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_pairs_kernel<kClass>, kThreads, smem);
   if (e != cudaSuccess) return e;
   const int64_t want = (a.p + (int64_t)kWarps * kBwdChunk - 1) / ((int64_t)kWarps * kBwdChunk);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)std::max(1, per_sm) * sm_count));
-  backward_fast_kernel<kNit><<<grid, kThreads, 0, st>>>(a);
+  backward_pairs_kernel<kClass><<<grid, kThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -511,15 +544,16 @@ cudaError_t launch_backward(const MapState& m, const float4* xyzl, int64_t p, co
   a.acc_class = acc_class;
   a.xyz_scale = (float)(m.prm.sigma0 / m.prm.length_scale);
   a.dc = m.dc;
-  if (2 * a.R + 1 <= kBwdAxis - 1) {
-    switch (a.tpad / 32) {  // unrolled sweeps for the common list lengths
-      case 2: return launch_backward_fast<2>(a, m.sm_count, m.stream);
-      case 3: return launch_backward_fast<3>(a, m.sm_count, m.stream);
-      case 4: return launch_backward_fast<4>(a, m.sm_count, m.stream);
-      case 5: return launch_backward_fast<5>(a, m.sm_count, m.stream);
-      case 6: return launch_backward_fast<6>(a, m.sm_count, m.stream);
-      default: return launch_backward_fast<0>(a, m.sm_count, m.stream);
-    }
+  // the pair form has its lists and addresses G with 32-bit element indices (and points for the re-decision)
+  if (m.ftab && (uint64_t)m.pool_blocks * (uint64_t)(m.g.K1 * m.g.B3) <= (1ull << 32) && p <= 0xffffffffll) {
+    a.ftab = m.ftab;
+    a.flen = m.flen;
+    a.list_pad = m.ftab_pad;
+    a.pad_list = m.ftab_pad_list;
+    a.fR = m.ftab_R;
+    a.band = 1.0625f * std::max(m.g.l2_hi - m.g.l2, m.g.l2 - m.g.l2_lo);
+    return acc_class ? launch_backward_pairs<true>(a, m.sm_count, m.stream)
+                     : launch_backward_pairs<false>(a, m.sm_count, m.stream);
   }
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_kernel, kThreads, 0);

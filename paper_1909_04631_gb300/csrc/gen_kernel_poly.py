@@ -98,6 +98,7 @@ def main():
     lines += horner("kernel_q", coefficients(Q, N), "Q(w), degree %d" % N)
     lines += horner2("kernel_q2", coefficients(Q, N), "Q(w), degree %d" % N)
     lines += horner("kernel_dq", coefficients(D, ND), "D(w), degree %d" % ND)
+    lines += horner2("kernel_dq2", coefficients(D, ND), "D(w), degree %d" % ND)
     lines += ["}  // namespace sbki", ""]
     out = os.path.join(os.path.dirname(os.path.abspath(__file__)), "kernel_poly.cuh")
     with open(out, "w") as fh:

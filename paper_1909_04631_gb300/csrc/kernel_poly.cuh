@@ -53,4 +53,21 @@ __device__ __forceinline__ float kernel_dq(float w) {
   return acc;
 }
 
+// D(w), degree 10, two arguments at once (packed FP32)
+__device__ __forceinline__ float2 kernel_dq2(float2 w) {
+  const float2 x = __ffma2_rn(make_float2(2.0f, 2.0f), w, make_float2(-1.0f, -1.0f));
+  float2 acc = make_float2(1.146870215e-07f, 1.146870215e-07f);
+  acc = __ffma2_rn(acc, x, make_float2(-2.831900989e-06f, -2.831900989e-06f));
+  acc = __ffma2_rn(acc, x, make_float2(5.735115500e-05f, 5.735115500e-05f));
+  acc = __ffma2_rn(acc, x, make_float2(-9.404646384e-04f, -9.404646384e-04f));
+  acc = __ffma2_rn(acc, x, make_float2(1.211086324e-02f, 1.211086324e-02f));
+  acc = __ffma2_rn(acc, x, make_float2(-1.182858189e-01f, -1.182858189e-01f));
+  acc = __ffma2_rn(acc, x, make_float2(8.361659899e-01f, 8.361659899e-01f));
+  acc = __ffma2_rn(acc, x, make_float2(-4.002633205e+00f, -4.002633205e+00f));
+  acc = __ffma2_rn(acc, x, make_float2(1.171144129e+01f, 1.171144129e+01f));
+  acc = __ffma2_rn(acc, x, make_float2(-1.752460235e+01f, -1.752460235e+01f));
+  acc = __ffma2_rn(acc, x, make_float2(9.086689068e+00f, 9.086689068e+00f));
+  return acc;
+}
+
 }  // namespace sbki

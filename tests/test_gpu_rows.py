@@ -81,3 +81,61 @@ def test_soft_labels(sb, orc, lr):
     with sb.Map(sb.default_params(**prm, track_pairs=1, pool_blocks=1 << 13, sample_capacity=1 << 16)) as m:
         st = m.insert_scan_soft(pts, probs, pose)
         assert st["pairs"] == _check(m, om, True)
+
+
+def _pairs_reference(prm, scale, xyz, lab, keys, G):
+    """FP64 gradients of sum G alpha, and a bound on the FP32 evaluation's error for each: per pair, with e = 2^-24, the
+    distance is within 4 e relative, u = 1 - d/l within 8 e, and the degree-10 (7) Horner form of the slope (kernel)
+    within 20 e (14 e) of its coefficients' absolute sum, 45 (9); a sum of n terms adds n e of its terms' magnitudes."""
+    e = 2.0 ** -24
+    l, s0, res = prm["length_scale"], prm["sigma0"], prm["res"]
+    c = (keys + 0.5) * res
+    gx, bx = np.zeros((len(xyz), 3)), np.zeros(len(xyz))
+    gl = gs = bl = bs = 0.0
+    gk, bk = np.zeros(len(scale)), np.zeros(len(scale))
+    for i, x in enumerate(xyz.astype(np.float64)):
+        o = c - x
+        d = np.sqrt((o[:, 0] ** 2 + o[:, 1] ** 2) + o[:, 2] ** 2)
+        m = (o[:, 0] ** 2 + o[:, 1] ** 2) + o[:, 2] ** 2 < l * l
+        o, d, g, s = o[m], d[m], G[m, lab[i]].astype(np.float64), scale[lab[i]]
+        u = 1 - d / l
+        f = (2 + np.cos(2 * np.pi * (1 - u))) * u / 3 + np.sin(2 * np.pi * (1 - u)) / (2 * np.pi)
+        df = (2 - 2 * np.cos(2 * np.pi * u)) / 3 - 2 * np.pi * u * np.sin(2 * np.pi * u) / 3  # -f'(r)
+        t = g * s0 * s * df / l
+        n = len(d) + 40
+        with np.errstate(all="ignore"):
+            gx[i] = (t[:, None] * np.where(d[:, None] > 0, o / d[:, None], 0)).sum(0)
+        bt = np.abs(g) * (u ** 4 * 900 * e + 4 * u ** 3 * 8 * e * 45 + 16 * e * np.abs(df))  # of g df
+        bf = np.abs(g) * (u ** 5 * 126 * e + 5 * u ** 4 * 8 * e * 9 + 16 * e * np.abs(f))    # of g f
+        bx[i] = s0 * s / l * (bt.sum() + n * e * np.abs(g * df).sum())
+        gs += s * (g * f).sum()
+        bs += s * (bf.sum() + n * e * np.abs(g * f).sum())
+        gl += s0 * s / l ** 2 * (g * df * d).sum()
+        bl += s0 * s / l ** 2 * l * (bt.sum() + n * e * np.abs(g * df).sum())
+        gk[lab[i]] += s0 * (g * f).sum()
+        bk[lab[i]] += s0 * (bf.sum() + n * e * np.abs(g * f).sum())
+    return gl, gs, gx, gk, bl, bs, bx, bk
+
+
+@pytest.mark.parametrize("lr,edge", [(0.6, 8), (0.87, 4), (1.5, 8), (2.5, 4), (3.0, 8), (3.0, 4), (3.45, 8), (3.6, 8)])
+@pytest.mark.parametrize("n", [1, 15, 17, 300])
+def test_backward_in_pairs(sb, lr, edge, n):
+    import torch
+    res, K = 0.1, 5
+    rng = np.random.default_rng(int(100 * lr) + edge + n)
+    xyz, lab = _cloud(rng, n, res, K + 1)
+    scale = [1.0, 0.5, 2.0, 1.25, 0.75, 1.0]
+    prm = dict(res=res, length_scale=lr * res, sigma0=0.4, alpha0=0.01, num_classes=K, block_edge=edge)
+    with sb.Map(sb.default_params(**prm, sigma0_scale=scale, pool_blocks=1 << 13, sample_capacity=1 << 14)) as m:
+        m.insert_training(xyz, lab)
+        keys, _, _ = m.export()
+        G = rng.normal(size=(len(keys), K + 1)).astype(np.float32)
+        m.grad_clear()
+        assert m.grad_add_alpha(keys, G) == 0
+        xyzl = torch.from_numpy(np.concatenate([xyz, lab[:, None].astype(np.float32)], 1)).cuda()
+        gl, gs, gx = m.backward(xyzl)
+        gk = m.backward_scales(xyzl)
+    rl, rs, rx, rk, bl, bs, bx, bk = _pairs_reference(prm, scale, xyz, lab, keys, G)
+    assert (np.abs(gx.cpu().numpy() - rx) <= bx[:, None] + 1e-12).all()
+    assert abs(gl - rl) <= bl + 1e-12 and abs(gs - rs) <= bs + 1e-12
+    assert (np.abs(gk - rk) <= bk + 1e-12).all()
