@@ -96,3 +96,35 @@ def test_query_points_street_training_set(sb, orc):
     got = sb.query_points(p, xyzl, q)
     want = orc.alpha_at_points(orc.params(**prm), x, lab, q.astype(np.float64))
     assert _rel(got, want).max() <= RTOL
+
+
+@pytest.mark.parametrize("n,spread,at,K", [(1, 0.01, 0.0, 1), (31, 0.05, 0.0, 31), (33, 0.05, -7.3, 31), (1024, 0.02, 3.0, 4),
+                                           (4097, 0.4, 850.0, 4), (70000, 1.5, -64.0, 11)])
+def test_query_points_runs_and_reach(sb, n, spread, at, K):
+    """Lists of one point to thousands per cell, around whole rounds of 32, every class count, near and far from the
+    origin, against the all-pairs FP64 sum.  Per pair, e = 2^-24: r = d / l is within 6 e, u = 1 - r within 8 e, the
+    kernel u^5 Q(u^2) within 16 e of itself, 126 e u^5 (its coefficients' absolute sum, 9, times 14 operations) and
+    5 u^4 8 e 9; a sum of n terms adds n e of it."""
+    rng = np.random.default_rng(n)
+    l, s0, a0, e = 0.3, 0.4, 0.001, 2.0 ** -24
+    xyz = (at + rng.normal(0, spread, size=(n, 3))).astype(np.float32)
+    lab = rng.integers(0, K + 1, size=n)
+    q = np.concatenate([xyz[rng.integers(0, n, 60)] + rng.normal(0, 0.15, size=(60, 3)),
+                        np.round(xyz[rng.integers(0, n, 40)] / (l * 1.001)) * (l * 1.001),  # corners of cells
+                        xyz[rng.integers(0, n, 20)] + l * np.eye(3)[rng.integers(0, 3, 20)]]).astype(np.float32)
+    p = sb.default_params(res=0.1, length_scale=l, sigma0=s0, alpha0=a0, num_classes=K, device=0)
+    xyzl = np.concatenate([xyz, lab[:, None].astype(np.float32)], 1)
+    got = sb.query_points(p, xyzl, q)
+    np.testing.assert_array_equal(sb.query_points(p, xyzl, q), got)  # the same order of the sums in every call
+    for i, x in enumerate(q.astype(np.float64)):
+        o = xyz.astype(np.float64) - x
+        d = np.sqrt((o * o).sum(1))
+        near = (o[:, 0] ** 2 + o[:, 1] ** 2) + o[:, 2] ** 2 < l * l
+        r = d[near] / l
+        f = (2 + np.cos(2 * np.pi * r)) * (1 - r) / 3 + np.sin(2 * np.pi * r) / (2 * np.pi)
+        u = 1 - r
+        b = 16 * e * f + 126 * e * u ** 5 + 5 * u ** 4 * 8 * e * 9
+        want, bound = np.full(K + 1, a0), np.full(K + 1, 4 * e * a0)
+        np.add.at(want, lab[near], s0 * f)
+        np.add.at(bound, lab[near], s0 * (b + (len(r) + 4) * e * f))
+        assert (np.abs(got[i] - want) <= bound).all()
