@@ -219,7 +219,8 @@ struct MapState {
   uint32_t ftab_classes = 0;            // classes with a table
   bool ftab_own_touched = false;        // every class's l above half the voxel diagonal (own block always touched)
   uint32_t* nbrslot = nullptr;          // fast form: [hash_cap][32] per own block (hash slot), the hash slots of the
-                                        // neighbour blocks its points touched in the last update, by block digit
+                                        // neighbour blocks its points touched in the last update, by block digit;
+                                        // entries 28, 29: the digits written in that update and its epoch
   float* gpool = nullptr;               // dL/dalpha [pool_blocks][K1][B3] (differentiable form, on first use)
   double* dacc = nullptr;               // [4 + 32]: held-out LL, sum s G f, sum s G u^4 D d, keys missed (as
                                         // u64), then sum G f per class

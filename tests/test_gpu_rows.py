@@ -139,3 +139,26 @@ def test_backward_in_pairs(sb, lr, edge, n):
     assert (np.abs(gx.cpu().numpy() - rx) <= bx[:, None] + 1e-12).all()
     assert abs(gl - rl) <= bl + 1e-12 and abs(gs - rs) <= bs + 1e-12
     assert (np.abs(gk - rk) <= bk + 1e-12).all()
+
+
+@pytest.mark.parametrize("lr,edge", [(0.87, 4), (0.87, 8), (2.0, 4), (3.0, 4), (3.0, 8), (3.5, 8)])
+@pytest.mark.parametrize("n", [1, 33, 2500])
+def test_touched_blocks_by_own_block(sb, lr, edge, n):
+    """The touched set of the point-major form (27 neighbour bits per own block) is the block-major form's, which walks
+    every point's candidate blocks: equal counts of touched and new blocks and equal blocks, over three updates."""
+    res, K = 0.1, 5
+    rng = np.random.default_rng(n + edge)
+    B = edge * res
+    prm = dict(res=res, length_scale=lr * res, sigma0=0.4, alpha0=0.001, num_classes=K, block_edge=edge,
+               pool_blocks=1 << 13, sample_capacity=1 << 14)
+    for assoc in (0, 1):
+        with sb.Map(sb.default_params(**prm, association=assoc)) as m, \
+                sb.Map(sb.default_params(**prm, association=assoc, accumulate_mode=1)) as b:
+            for _ in range(3):
+                xyz, lab = _cloud(rng, n, res, K + 1)
+                xyz[::3] = (np.round(xyz[::3] / B) * B + rng.choice([-1, 0, 1], size=xyz[::3].shape)
+                            * lr * res * rng.choice([0.5, 1.0, 2 ** -0.5], size=(len(xyz[::3]), 1))).astype(np.float32)
+                sm, sbl = m.insert_training(xyz, lab), b.insert_training(xyz, lab)
+                assert sm["touched_blocks"] == sbl["touched_blocks"] and sm["new_blocks"] == sbl["new_blocks"]
+            km, kb = m.export()[0], b.export()[0]
+            np.testing.assert_array_equal(km, kb)
