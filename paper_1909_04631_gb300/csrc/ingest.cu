@@ -818,14 +818,16 @@ cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n) {
   return cudaGetLastError();
 }
 
+// The per-point counts become output offsets.
+cudaError_t launch_offsets(MapState& m, int64_t total_n) {
+  m.launches += 1;
+  return exclusive_scan_u64_onepass(m.s.cnt, total_n, m.s.scan_tmp, m.stream, &m.dc->n_scan, m.sm_count, m.dc);
+}
+
 cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, uint32_t* hit_src) {
   const int64_t warps = (total_n + 7) / 8;
   unsigned blocks = (unsigned)std::min<int64_t>((warps + 7) / 8, (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm);
   if (blocks == 0) blocks = 1;
-  // the per-point counts become output offsets
-  cudaError_t e = exclusive_scan_u64_onepass(m.s.cnt, total_n, m.s.scan_tmp, m.stream, &m.dc->n_scan, m.sm_count, m.dc);
-  if (e != cudaSuccess) return e;
-  m.launches += 1;
   emit_kernel<<<blocks, 256, 0, m.stream>>>(m.s.world, m.s.cnt, m.s.desc, ns, m.g, kf, m.s.items, m.s.keys, m.s.vals,
                                             hit_src, m.dc);
   m.launches += 1;

@@ -482,6 +482,7 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   // back, so the read-back also tells how many are occupied.
   const bool marked = !probs && tile_frame_fits(m, 1, kf);
   if (marked) CK(&m, launch_tile_mark(m, 1, n, kf));
+  if (probs) CK(&m, launch_offsets(m, n));  // the sorted form for certain: while the host waits
   st = read_counters(m);
   if (st != SBKI_OK) return st;
   if (m.hc->err != 0) return status_from_device(m);
@@ -504,6 +505,7 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
     CK(&m, launch_tiles(m, 1, n, kf, *nitems));
     return SBKI_OK;
   }
+  if (!probs) CK(&m, launch_offsets(m, n));
   CK(&m, launch_emit(m, 1, n, kf, probs ? m.s.hit_src : nullptr));
   CK(&m, launch_downsample_n(m, kf, *nitems));
   if (probs) CK(&m, launch_soft_weights(m));
@@ -951,6 +953,7 @@ sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t cou
       ce = launch_tile_mark(m, count, m.s.n_cap, kf);
       if (ce == cudaSuccess) ce = launch_tiles(m, count, m.s.n_cap, kf, m.s.s_cap);
     }
+    if (ce == cudaSuccess) ce = launch_offsets(m, m.s.n_cap);
     if (ce == cudaSuccess) ce = launch_emit(m, count, m.s.n_cap, kf);
     if (ce == cudaSuccess) ce = launch_downsample_n(m, kf, m.s.s_cap);
     sbki_status ust = SBKI_OK;

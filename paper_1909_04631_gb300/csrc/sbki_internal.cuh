@@ -367,6 +367,8 @@ cudaError_t radix_wait_selftest(unsigned long long* keys, uint32_t* vals, unsign
 // ingest.cu
 // ingest of the ns scans described in m.s.desc (ns + 1 entries, the last holding the total)
 cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n);
+// sorted form: the points' counts to offsets (the tile form reads the counts), then the items
+cudaError_t launch_offsets(MapState& m, int64_t total_n);
 cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, uint32_t* hit_src = nullptr);
 cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems);
 // tiles.cu: the downsampling by occupied tiles.  The frame must fit the
