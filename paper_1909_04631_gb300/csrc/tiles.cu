@@ -276,7 +276,12 @@ struct MarkOp {
   }
 };
 __global__ void __launch_bounds__(256, 6) tile_mark_kernel(TileArgs a) {
-  if (a.dc->err) return;  // uniform: written before this launch, or to the same value below
+  // make_item of this launch may set the error while other CTAs start, so one read decides for the whole CTA:
+  // warps that went on without the others would miss each_item's scan offsets
+  __shared__ int s_err;
+  if (threadIdx.x == 0) s_err = *(volatile const int*)&a.dc->err;
+  __syncthreads();
+  if (s_err) return;
   MarkOp op{a};
   each_item(a, op);
   const uint32_t w = __reduce_add_sync(0xffffffffu, op.fresh);

@@ -98,3 +98,23 @@ def test_errors_and_recovery(sb):
         assert e.value.status == sb.ERR_CAPACITY
         st = m.insert_scan(pts, lab, np.eye(4))
         assert st["hits"] == 500 and st["train_points"] > 0
+
+
+def test_items_outside_the_frame_of_a_batch_are_refused(sb):
+    """A pose whose 3x3 part scales by ten puts items outside the frame of max_range on every side: a batch says so
+    (the error is set while CTAs of the same launch still start), no map changes, and the handle works after."""
+    rng = np.random.default_rng(11)
+    pts = rng.uniform(-9, 9, (3000, 3)).astype(np.float32)
+    lab = np.ones(len(pts), np.int32)
+    wide = np.eye(4)
+    wide[:3, :3] *= 10
+    with sb.Map(sb.default_params(num_classes=3, max_range=50.0, pool_blocks=1 << 15, sample_capacity=1 << 22)) as m:
+        m.insert_batch([dict(points=pts, labels=lab, pose=np.eye(4), map_id=0)] * 2)
+        before = m.export()
+        with pytest.raises(sb.SbkiError) as e:
+            m.insert_batch([dict(points=pts, labels=lab, pose=T, map_id=0) for T in (np.eye(4), wide)])
+        assert e.value.status == sb.ERR_INVALID_ARG
+        for a, b in zip(before[:2], m.export()[:2]):
+            np.testing.assert_array_equal(a, b)
+        st = m.insert_scan(pts, lab, np.eye(4))
+        assert st["hits"] == len(pts)
