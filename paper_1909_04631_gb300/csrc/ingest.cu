@@ -105,7 +105,9 @@ __device__ __forceinline__ unsigned long long transform_count_one(const ScanDesc
       w = make_float4(wc[0], wc[1], wc[2], (float)lab);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const int t = floor_i(__fmul_rn(wc[a], g.inv_ds)) >> kTileShift;
+        const float q = __fmul_rn(wc[a], g.inv_ds);
+        const int t = floor_i(q) >> kTileShift;
+        if (!(fabsf(q) < 4194304.0f)) atomicMax(&dc->n_ttiles, kTilesDeclined);  // no rigid pose reaches that far
         tlo[a] = min(tlo[a], t);
         thi[a] = max(thi[a], t);
       }

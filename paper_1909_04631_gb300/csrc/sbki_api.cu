@@ -479,9 +479,10 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   CK(&m, launch_transform_count(m, 1, n));
   // The tile form (soft labels need the sorted items).  Where the frame of
   // max_range fits a directory, the tiles are marked before the counters come
-  // back, so the read-back also tells how many are occupied.
+  // back, so the read-back also tells how many are occupied (or that items lie
+  // outside: a pose that scales or shears; the fitted frame below holds them).
   const bool marked = !probs && tile_frame_fits(m, 1, kf);
-  if (marked) CK(&m, launch_tile_mark(m, 1, n, kf));
+  if (marked) CK(&m, launch_tile_mark(m, 1, n, kf, false));
   if (probs) CK(&m, launch_offsets(m, n));  // the sorted form for certain: while the host waits
   st = read_counters(m);
   if (st != SBKI_OK) return st;
@@ -493,15 +494,16 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
     return SBKI_OK;
   }
   fit_frame_to_box(m.g, m.hc->tbox, T, kf);
+  if (kf.total_bits > 64) return fail(&m, SBKI_ERR_INVALID_ARG, "scan spans too large a region");
   for (int a = 0; a < 3; ++a) {
     m.hdesc[0].org[a] = kf.org[a];
     m.hdesc[0].ext[a] = kf.ext[a];
   }
   CK(&m, cudaMemcpyAsync(m.s.desc, m.hdesc, sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
   // a frame fitted to the hits that cannot hold more tiles than there is room for
-  if (!probs && !marked && tile_frame_fits(m, 1, kf) && tile_items_fit(m, *nitems) &&
+  if (!probs && !marked && m.hc->n_ttiles < kTilesDeclined && tile_frame_fits(m, 1, kf) && tile_items_fit(m, *nitems) &&
       std::min<int64_t>((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2], *nitems) <= tile_capacity(m.s.s_cap)) {
-    CK(&m, launch_tile_mark(m, 1, n, kf));
+    CK(&m, launch_tile_mark(m, 1, n, kf, true));
     CK(&m, launch_tiles(m, 1, n, kf, *nitems));
     return SBKI_OK;
   }
@@ -950,7 +952,7 @@ sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t cou
     cudaError_t ce = launch_transform_count(m, count, m.s.n_cap);
     // the tile form where the scans' frames fit, then the sorted form for what it leaves (as a rule nothing)
     if (ce == cudaSuccess && tile_frame_fits(m, count, kf)) {
-      ce = launch_tile_mark(m, count, m.s.n_cap, kf);
+      ce = launch_tile_mark(m, count, m.s.n_cap, kf, false);
       if (ce == cudaSuccess) ce = launch_tiles(m, count, m.s.n_cap, kf, m.s.s_cap);
     }
     if (ce == cudaSuccess) ce = launch_offsets(m, m.s.n_cap);

@@ -56,7 +56,7 @@ struct DevCounters {
   uint32_t n_scan;                    // points whose sample counts it sums up (likewise)
   uint32_t transform_done;            // CTAs of the transform finished (the last one adds up the counts)
   unsigned long long n_total;         // hits << 40 | free samples of this scan
-  uint32_t n_ttiles;                  // tile form: occupied tiles
+  uint32_t n_ttiles;                  // tile form: occupied tiles (kTilesDeclined and more: not this form)
   uint32_t n_low;                     // tile form: fractions noted
   uint32_t n_wide;                    // tile form: training points left to the gathered exact mean
   uint32_t n_gather;                  // tile form: their members
@@ -374,11 +374,13 @@ cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems)
 // tiles.cu: the downsampling by occupied tiles.  The frame must fit the
 // scratch (tile_frame_fits), the items leave room for the flagged points
 // (tile_items_fit), and the occupied tiles not exceed tile_capacity.
+constexpr uint32_t kTilesDeclined = 1u << 30;  // an item outside the frame, or in a cell beyond 2^22
 constexpr int64_t kTileFrameMax = 1 << 22;  // directory entries per scan at most
 int64_t tile_capacity(int64_t sample_capacity);
 bool tile_frame_fits(const MapState& m, int ns, const KeyFrame& kf);
 bool tile_items_fit(const MapState& m, int64_t nitems);
-cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf);
+// alone: the sorted form does not follow, an item outside the frame is an error; else it declines the tile form
+cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, bool alone);
 cudaError_t launch_tiles(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, int64_t nitems);
 cudaError_t launch_train_bbox(MapState& m, const float4* in, int64_t p, int* bbox_dev);
 cudaError_t launch_train_prepare(MapState& m, const float4* in, int64_t p, const KeyFrame& kf);

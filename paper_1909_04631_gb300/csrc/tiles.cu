@@ -89,6 +89,7 @@ struct TileArgs {
   int ns;
   float4* train;
   DevCounters* dc;
+  bool alone;           // no sorted form behind: an item outside the frame is an error
   uint32_t pack_limit;  // scans of fewer points have no cell of 2^19 members: counts ride on the sums
 };
 
@@ -113,11 +114,12 @@ struct Item {
   float x[3];
   int gc[3];  // downsampling cell per axis
   uint32_t entry, cell;  // cell | label << kLocalBits
+  bool out;              // live, but outside the frame (no entry)
   __device__ __forceinline__ uint32_t local() const { return cell & (uint32_t)(kCells - 1); }
   __device__ __forceinline__ uint32_t label() const { return cell >> kLocalBits; }
 };
 __device__ __forceinline__ Item make_item(bool live, float x, float y, float z, uint32_t label, const Geom& g,
-                                          const TileFrame& f, DevCounters* dc) {
+                                          const TileFrame& f) {
   Item it;
   it.x[0] = x;
   it.x[1] = y;
@@ -126,18 +128,16 @@ __device__ __forceinline__ Item make_item(bool live, float x, float y, float z, 
   bool in = true;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    it.gc[a] = floor_small(__fmul_rn(it.x[a], g.inv_ds));  // |cell| < 2^22 (tile_frame_fits)
+    it.gc[a] = floor_small(__fmul_rn(it.x[a], g.inv_ds));  // |cell| < 2^22 (the transform declines others)
     t[a] = (it.gc[a] >> kTileShift) - f.o[a];
     in = in && (uint32_t)t[a] < (uint32_t)f.e[a];
   }
   constexpr int m = kTileEdge - 1;
   it.cell = (uint32_t)(((it.gc[2] & m) << (2 * kTileShift)) | ((it.gc[1] & m) << kTileShift) | (it.gc[0] & m)) |
             label << kLocalBits;
+  it.out = live && !in;
   it.entry = kNoPoint;
-  if (live) {
-    if (in) it.entry = f.first + (uint32_t)((t[0] * f.e[1] + t[1]) * f.e[2] + t[2]);
-    else set_error(dc, SBKI_ERR_INVALID_ARG);
-  }
+  if (live && in) it.entry = f.first + (uint32_t)((t[0] * f.e[1] + t[1]) * f.e[2] + t[2]);
   return it;
 }
 
@@ -219,7 +219,7 @@ __device__ __forceinline__ void each_item(const TileArgs& a, Op& op) {
       w = a.world[i];
     }
     if (phase == 0) {
-      const Item it = make_item(hit, w.x, w.y, w.z, (uint32_t)(int)w.w, g, f, a.dc);
+      const Item it = make_item(hit, w.x, w.y, w.z, (uint32_t)(int)w.w, g, f);
       op.apply(op.look(it, Run(it)));
     }
     const float sx = __fsub_rn(w.x, o[0]), sy = __fsub_rn(w.y, o[1]), sz = __fsub_rn(w.z, o[2]);
@@ -234,7 +234,7 @@ __device__ __forceinline__ void each_item(const TileArgs& a, Op& op) {
         const bool live = j <= nfree;
         const float k = by_r(__fsub_rn(rr, __fmul_rn((float)j, g.step)));
         const Item it = make_item(live, __fadd_rn(o[0], __fmul_rn(sx, k)), __fadd_rn(o[1], __fmul_rn(sy, k)),
-                                  __fadd_rn(o[2], __fmul_rn(sz, k)), 0u, g, f, a.dc);
+                                  __fadd_rn(o[2], __fmul_rn(sz, k)), 0u, g, f);
         found[u] = op.look(it, Run(it));
       }
 #pragma unroll
@@ -257,10 +257,12 @@ struct MarkOp {
   };
   const TileArgs& a;
   uint32_t fresh = 0;
+  bool out = false;
   // A tile's word is mostly set already: a cached read first (it may be an old
   // 0), then one past the L1, so the tiles around the sensor do not serialise.
-  __device__ __forceinline__ Found look(const Item& it, const Run& run) const {
+  __device__ __forceinline__ Found look(const Item& it, const Run& run) {
     Found f{it.entry, 1u};
+    out = out || it.out;
     if (run.last && it.entry != kNoPoint) {
       f.old = a.b.dir[it.entry];
       if (f.old == 0u) f.old = *(volatile const uint32_t*)(a.b.dir + it.entry);
@@ -276,16 +278,22 @@ struct MarkOp {
   }
 };
 __global__ void __launch_bounds__(256, 6) tile_mark_kernel(TileArgs a) {
-  // make_item of this launch may set the error while other CTAs start, so one read decides for the whole CTA:
-  // warps that went on without the others would miss each_item's scan offsets
-  __shared__ int s_err;
-  if (threadIdx.x == 0) s_err = *(volatile const int*)&a.dc->err;
+  // other CTAs of this launch may set the error or decline, so one read decides for the whole CTA: warps that
+  // went on without the others would miss each_item's scan offsets
+  __shared__ int s_off;
+  if (threadIdx.x == 0)
+    s_off = *(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles >= kTilesDeclined;
   __syncthreads();
-  if (s_err) return;
+  if (s_off) return;
   MarkOp op{a};
   each_item(a, op);
   const uint32_t w = __reduce_add_sync(0xffffffffu, op.fresh);
+  const bool out = __any_sync(0xffffffffu, op.out);
   if ((threadIdx.x & 31) == 0 && w) atomicAdd(&a.dc->n_ttiles, w);
+  if ((threadIdx.x & 31) == 0 && out) {  // a pose that scales or shears can leave the frame of max_range
+    if (a.alone) set_error(a.dc, SBKI_ERR_INVALID_ARG);
+    else atomicMax(&a.dc->n_ttiles, kTilesDeclined);
+  }
 }
 
 // The scan whose directory entries hold e, and e's tile per axis.
@@ -750,7 +758,7 @@ unsigned item_blocks(const MapState& m, int64_t total_n) {
       1, std::min<int64_t>(((total_n + 31) / 32 * kPhases + 7) / 8, (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm));
 }
 
-TileArgs tile_args(const MapState& m, int ns, uint32_t entries) {
+TileArgs tile_args(const MapState& m, int ns, uint32_t entries, bool alone) {
   const Scratch& s = m.s;
   TileArgs a;
   a.g = m.g;
@@ -779,6 +787,7 @@ TileArgs tile_args(const MapState& m, int ns, uint32_t entries) {
   a.ns = ns;
   a.train = s.train;
   a.dc = m.dc;
+  a.alone = alone;
   a.b.item_cap = (uint32_t)std::max<int64_t>(0, s.s_cap - 5 * (int64_t)a.b.tile_cap - 1);
   // a beam's samples lie `step` apart, so at most 1 + sqrt(3) ds / step of them are in one cell
   // (widened for FP32 positions); a point's members are hits (one a beam) or samples, never both
@@ -810,9 +819,9 @@ bool tile_items_fit(const MapState& m, int64_t nitems) {
   return nitems + 5 * tile_capacity(m.s.s_cap) + 1 <= m.s.s_cap;
 }
 
-cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf) {
+cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, bool alone) {
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
-  const TileArgs a = tile_args(m, ns, entries);
+  const TileArgs a = tile_args(m, ns, entries, alone);
   cudaError_t e = cudaMemsetAsync(a.b.dir, 0, sizeof(uint32_t) * (size_t)directory_words(entries, a.b.tile_cap), m.stream);
   if (e != cudaSuccess) return e;
   tile_mark_kernel<<<item_blocks(m, total_n), 256, 0, m.stream>>>(a);
@@ -822,7 +831,7 @@ cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFram
 
 cudaError_t launch_tiles(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, int64_t nitems) {
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
-  const TileArgs a = tile_args(m, ns, entries);
+  const TileArgs a = tile_args(m, ns, entries, false);
   const unsigned blocks = item_blocks(m, total_n);
   const int64_t sms = m.sm_count;
   tile_rank_kernel<<<(unsigned)std::min<int64_t>(entries / kChunk + 1, 8 * sms), 256, 0, m.stream>>>(a);

@@ -118,3 +118,68 @@ def test_items_outside_the_frame_of_a_batch_are_refused(sb):
             np.testing.assert_array_equal(a, b)
         st = m.insert_scan(pts, lab, np.eye(4))
         assert st["hits"] == len(pts)
+
+
+def _affine(kind):
+    T = _pose(0.4, -0.3, 0.2, 0.7)
+    if kind == "scaled":
+        T[:3, :3] *= 8
+    elif kind == "sheared":
+        T[:3, :3] = T[:3, :3] @ np.array([[5.0, 3.0, 0], [0, 6.0, -2.0], [0, 0, 7.0]])
+    elif kind == "mirrored":
+        T[:3, :3] = T[:3, :3] @ np.diag([-9.0, 1.0, 1.0])
+    else:  # "far": one axis beyond 2^22 cells
+        T = np.eye(4)
+        T[0, 0] = 1e5
+    return T
+
+
+@pytest.mark.parametrize("kind", ["scaled", "sheared", "mirrored", "far"])
+def test_poses_that_leave_the_frame_of_max_range(sb, orc, kind):
+    """A pose is any affine transform: hits within max_range of the sensor may lie further off in the world.  The
+    training set is the oracle's, whether the frame of max_range fits the directory (50 m) or not (400 m)."""
+    rng = np.random.default_rng(len(kind))
+    T = _affine(kind)
+    if kind == "far":
+        pts = np.array([[5.0, 0.7, -0.6]], np.float32)
+    else:
+        pts = rng.uniform(-9, 9, (1500, 3)).astype(np.float32)
+    lab = rng.integers(1, 4, len(pts)).astype(np.int32)
+    for max_range in (50.0, 400.0):
+        prm = dict(res=0.1, length_scale=0.3, sigma0=0.4, alpha0=0.001, free_step=0.3, num_classes=3, max_range=max_range)
+        ox, ol, st = orc.training_set(orc.params(**prm), pts, lab, T)
+        with sb.Map(sb.default_params(**prm, pool_blocks=1 << 12, sample_capacity=1 << 22)) as m:
+            gx, gl = m.training_set(pts, lab, T)
+        assert len(gx) == st["train"]
+        o, g = np.lexsort((ol, *ox.T)), np.lexsort((gl, *gx.T))
+        np.testing.assert_array_equal(gl[g], ol[o])
+        np.testing.assert_array_equal(gx[g], ox[o])
+
+
+def test_a_scan_too_wide_for_the_keys_is_refused(sb):
+    pts = np.array([[5.0, 5.0, 5.0]], np.float32)
+    T = np.diag([1e5, 1e5, 1e5, 1.0])
+    for max_range in (50.0, 400.0):
+        with sb.Map(sb.default_params(num_classes=3, max_range=max_range, pool_blocks=1 << 12, sample_capacity=1 << 22)) as m:
+            with pytest.raises(sb.SbkiError) as e:
+                m.training_set(pts, np.ones(1, np.int32), T)
+            assert e.value.status == sb.ERR_INVALID_ARG
+            assert len(m.training_set(pts, np.ones(1, np.int32), np.eye(4))[0]) > 0
+
+
+def test_batch_with_items_past_the_frame_but_within_the_keys(sb):
+    """Tiles are counted up to the frame of max_range (131 per axis here), keys hold 256: a batch with items between
+    the two is taken, as two updates would be."""
+    rng = np.random.default_rng(5)
+    prm = dict(num_classes=3, max_range=50.0, pool_blocks=1 << 16, sample_capacity=1 << 22, track_pairs=1)
+    wide = np.diag([8.0, 8.0, 8.0, 1.0])
+    scans = [dict(points=rng.uniform(1, 9, (300, 3)).astype(np.float32), labels=np.ones(300, np.int32), pose=T, map_id=0)
+             for T in (wide, np.eye(4))]
+    with sb.Map(sb.default_params(**prm)) as mb, sb.Map(sb.default_params(**prm)) as ms:
+        mb.insert_batch(scans)
+        for s in scans:
+            ms.insert_scan(s["points"], s["labels"], s["pose"])
+        (kb, ab, pb), (ks, as_, ps) = mb.export(pairs=True), ms.export(pairs=True)
+    np.testing.assert_array_equal(kb, ks)
+    np.testing.assert_array_equal(pb, ps)
+    np.testing.assert_allclose(ab, as_, rtol=1e-5)  # sums in another order
