@@ -495,11 +495,16 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   }
   fit_frame_to_box(m.g, m.hc->tbox, T, kf);
   if (kf.total_bits > 64) return fail(&m, SBKI_ERR_INVALID_ARG, "scan spans too large a region");
+  // Staged apart from hdesc[0]: an asynchronous update returns with this copy in
+  // flight and the next one writes hdesc[0] at once.  It comes here only after
+  // its own read-back, which waits for this copy.
+  ScanDesc& fitted = m.hdesc[kMaxScans + 1];
+  fitted = m.hdesc[0];
   for (int a = 0; a < 3; ++a) {
-    m.hdesc[0].org[a] = kf.org[a];
-    m.hdesc[0].ext[a] = kf.ext[a];
+    fitted.org[a] = kf.org[a];
+    fitted.ext[a] = kf.ext[a];
   }
-  CK(&m, cudaMemcpyAsync(m.s.desc, m.hdesc, sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
+  CK(&m, cudaMemcpyAsync(m.s.desc, &fitted, sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
   // a frame fitted to the hits that cannot hold more tiles than there is room for
   if (!probs && !marked && m.hc->n_ttiles < kTilesDeclined && tile_frame_fits(m, 1, kf) && tile_items_fit(m, *nitems) &&
       std::min<int64_t>((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2], *nitems) <= tile_capacity(m.s.s_cap)) {
@@ -725,7 +730,7 @@ sbki_status sbki_create_map(const sbki_params* params, sbki_map** out) {
   if ((ce = cudaMalloc(&s.carry, (size_t)kSegCarryBytes * 2 * seg_tiles(S))) != cudaSuccess)
     return bail("segment carries", ce);
   if ((ce = dalloc(&s.desc, kMaxScans + 1)) != cudaSuccess) return bail("scan descriptors", ce);
-  if ((ce = cudaMallocHost((void**)&m.hdesc, sizeof(ScanDesc) * (kMaxScans + 1))) != cudaSuccess)
+  if ((ce = cudaMallocHost((void**)&m.hdesc, sizeof(ScanDesc) * (kMaxScans + 2))) != cudaSuccess)
     return bail("host scan descriptors", ce);
   if ((ce = dalloc(&s.fresh, m.hash_cap)) != cudaSuccess) return bail("fresh list", ce);
   if ((ce = cudaMemsetAsync(m.hkeys, 0xff, sizeof(unsigned long long) * m.hash_cap, m.stream)) != cudaSuccess)

@@ -206,7 +206,7 @@ struct MapState {
   int64_t batch_kernels[kMaxScans + 1] = {};       // kernels in each recording
   uint64_t batch_gen[kMaxScans + 1] = {};          // scratch generation each recording used
   uint64_t scratch_gen = 1;             // advances when scratch buffers move
-  ScanDesc* hdesc = nullptr;            // pinned host staging of s.desc
+  ScanDesc* hdesc = nullptr;            // pinned host staging of s.desc; entry kMaxScans + 1: a scan's fitted frame
   uint32_t* ctab = nullptr;             // point-major candidate lists [kParts^3][ctab_pad]
   int32_t* clen = nullptr;              // [kParts^3] entries of each list
   uint16_t* ftab = nullptr;             // fast accumulation form's candidate lists (2R + 1 <= 7), or null:

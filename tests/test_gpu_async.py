@@ -93,3 +93,33 @@ def test_async_error_surfaces_and_leaves_the_map_unchanged(sb, scans):
         after = m.export(pairs=True)
         for a, b in zip(before, after):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("form", ["tiles", "sorted"])
+def test_back_to_back_inserts_keep_their_own_descriptors(sb, form):
+    """A frame fitted to the hits (max_range too large for the directory) is sent to the device after the counters
+    came back and the call returns with that copy in flight: forty inserts issued without a wait, alternating
+    between two scans of other sizes, poses and boxes, equal forty waited for."""
+    import torch
+    rng = np.random.default_rng(2)
+    scans = []
+    for n, half, at in ((2000, 3.0, (0.0, 0.0, 0.0)), (300, 14.0, (40.0, -25.0, 3.0))):
+        T = np.eye(4)
+        T[:3, 3] = at
+        scans.append((torch.from_numpy(rng.uniform(-half, half, (n, 3)).astype(np.float32)).cuda(),
+                      torch.ones(n, dtype=torch.int32, device="cuda"), T))
+    # the sorted form: a scratch with room for the items but not for as many flagged points and tiles
+    cap = 1 << 21 if form == "tiles" else 20800
+    prm = sb.default_params(res=0.1, length_scale=0.3, num_classes=3, max_range=400.0, pool_blocks=1 << 16,
+                            sample_capacity=cap, track_pairs=1, device=0)
+    with sb.Map(prm) as ma, sb.Map(prm) as ms:
+        for i in range(40):
+            p, l, T = scans[i % 2]
+            ma.insert_scan(p, l, T, sync=False)
+            ms.insert_scan(p, l, T)
+        ma.sync()
+        ka, aa, pa = ma.export(pairs=True)
+        ks, as_, ps = ms.export(pairs=True)
+    np.testing.assert_array_equal(ka, ks)
+    np.testing.assert_array_equal(pa, ps)
+    assert _rel(aa, as_).max() <= 1e-5
