@@ -343,9 +343,17 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
       const int gn = (int)min(c1 - g0, (int64_t)kGroup);  // warp-uniform
       // rows of every point of the group, four lanes per point
       int pt = 0, lw = 0, b0 = 0;
+      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (gl < gn) p = a.xyzl[g0 + gl];
+      float x = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
+      // A coordinate that is not finite or past floor_small's range reaches no voxel of a map.  Every candidate is
+      // multiplied out below, masked or not, so such a point's rows must not hold it (0 * inf is NaN): they are formed
+      // at 0 and the point takes no list.
+      const bool inside = fabsf(__fmul_rn(x, g.inv_res)) < 4194304.0f;
+      const uint32_t insides = __ballot_sync(0xffffffffu, inside);
+      if (!inside) x = 0.f;
       if (gl < gn) {
-        const float4 p = a.xyzl[g0 + gl];
-        const AxisFrame f = axis_frame(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), g);
+        const AxisFrame f = axis_frame(x, g);
         lw = label_of(p.w);
         pt = form_rows<false>(W.slot[gl], gl, role, f, (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3), R, g);
         b0 = f.v0 >> g.B_shift;
@@ -355,7 +363,8 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
       if (role == 0 && gl < gn) {
         const int list = pt + kFastParts * (pty + kFastParts / 2 * ptz);
         const int label = lw & ((1 << kLabelBits) - 1), map = lw >> kLabelBits;
-        const bool known = label < g.K1 && map < kMaxMaps;  // others have no G
+        // others have no G
+        const bool known = label < g.K1 && map < kMaxMaps && ((insides >> lane) & 15u) == 15u;
         const unsigned long long key = known ? pack_block(b0, by, bz, map) : kEmpty;
         uint32_t* sc = reinterpret_cast<uint32_t*>(W.slot[gl] + kScalars);
         sc[0] = known ? (uint32_t)(list * a.list_pad) : a.pad_list;

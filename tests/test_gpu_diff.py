@@ -201,3 +201,36 @@ def test_gradient_with_class_scales_matches_oracle(sb, orc, diff_case):
     assert np.all(gsc[~used] == 0)
     # the scaling identity holds on the GPU too
     assert float(np.dot(scale, gsc)) == pytest.approx(c["prm"]["sigma0"] * gs, rel=1e-6)
+
+
+@pytest.mark.parametrize("lr", [3.0, 4.5])  # pairs of voxels, one voxel per lane
+def test_points_that_reach_no_voxel_add_nothing(sb, diff_case, lr):
+    """Points with a coordinate that is not finite, overflows when squared or lies beyond every map, among the points
+    of a set: the sums over the set are those without them (every term here has the sign of the others, and the sums
+    hold 2^-40 or better), the other rows of dL/dxyz keep their bits, theirs are zero."""
+    c = diff_case
+    p = _params(sb, c["prm"], length_scale=lr * c["prm"]["res"])
+    n = 1000
+    xyz, lab = c["xyz"][:n], c["lab"][:n]
+    xyzl = np.concatenate([xyz, lab[:, None].astype(np.float32)], 1)
+    bad = np.float32([[v if a == ax else 0.3 for a in range(3)] for ax in range(3)
+                      for v in (np.nan, np.inf, -np.inf, 1e30, -3e38, 2e19, 5e6)])
+    bad = np.concatenate([bad, np.float32([[np.nan] * 3, [np.inf, -np.inf, np.nan]])])
+    bad = np.concatenate([bad, np.full((len(bad), 1), lab[0], np.float32)], 1)
+    at = np.sort(np.concatenate([[0, 1, n, n], np.random.default_rng(4).integers(2, n, len(bad) - 4)]))
+    both = np.insert(xyzl, at, bad, axis=0)
+    is_bad = np.insert(np.zeros(n, bool), at, True)
+    with sb.Map(p) as m:
+        m.insert_training(xyz, lab)
+        m.grad_clear()
+        keys, alpha, _ = m.export()
+        assert m.grad_add_alpha(keys, np.ones(alpha.shape, np.float32)) == 0
+        gl, gs, gx = m.backward(xyzl)
+        sc = m.backward_scales(xyzl)
+        gl2, gs2, gx2 = m.backward(both)
+        sc2 = m.backward_scales(both)
+    assert gl != 0 and gs > 0
+    assert abs(gl2 - gl) <= 2.0**-38 * abs(gl) and abs(gs2 - gs) <= 2.0**-38 * gs
+    np.testing.assert_allclose(sc2, sc, rtol=2.0**-20)  # a point's sum by class is taken in FP32
+    np.testing.assert_array_equal(gx2[~is_bad], gx)
+    np.testing.assert_array_equal(gx2[is_bad], 0)
