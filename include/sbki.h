@@ -342,8 +342,10 @@ sbki_status sbki_grad_add_alpha(sbki_map* map, const int64_t* keys, const float*
  *   grad_sigma0 = sum G f(r),  grad_l = sum G sigma0 f'(r) (-d/l^2),
  *   grad_xyz[i] = sum_v G sigma0 f'(r) (x_i - c_v)/(l d)   ([p,3], nullable,
  *   host or device; 0 where d = 0).
- * grad_l and grad_sigma0 (host, nullable) are summed in FP64 from FP32 pair
- * terms.  A counting-model map (piecewise constant in x, no l or sigma0)
+ * grad_l and grad_sigma0 (host, nullable) are sums of FP32 pair terms: a
+ * point's terms in FP32, points in unevaluated FP32 pairs of 2^-44 relative
+ * (at most 32 points) or in FP64, and the rest in FP64.  A training point
+ * with a coordinate that is not finite adds nothing.  A counting-model map (piecewise constant in x, no l or sigma0)
  * returns SBKI_ERR_INVALID_ARG. */
 sbki_status sbki_backward(sbki_map* map, const float* xyzl, int64_t p, double* grad_l, double* grad_sigma0,
                           float* grad_xyz);

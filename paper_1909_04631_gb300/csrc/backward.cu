@@ -264,15 +264,18 @@ __global__ void __launch_bounds__(kThreads, 3) backward_kernel(BwdArgs a) {
 // a warp per point, two voxels adjacent in x per lane; the rows hold the offsets
 // themselves here), for supports of at most 7 offsets per axis.  A pair reads
 // its two values of G in one 8-byte load; kernel, slope and the sums are packed
-// FP32.  FP64 runs at 1/64 of the FP32 rate on this chip, so the sums over the
-// points are unevaluated FP32 pairs per lane (error-free sums and products, so
-// as accurate as FP64), joined in FP64 once per warp.
+// FP32.  FP64 runs at 1/64 of the FP32 rate on this chip, so a lane sums the
+// points of a few chunks as unevaluated FP32 pairs (error-free sums and
+// products, 2^-44 relative over its 32 points) and then adds them to an FP64
+// sum: neither the range nor the error depends on the length of the set (after
+// every chunk it costs 1 % more).
 //
 // Bound by instruction issue, as the accumulation's sweep is.  2.0M points,
 // 223M pairs: one voxel per lane with FP64 sums per point took 1378 us, this
 // form takes 905.  The largest part of the difference are the FP64 sums: two
 // fused multiply-adds per point and lane hold the SM's FP64 units for ~900 us.
 constexpr int kBwdChunk = 16;  // consecutive training points per warp
+constexpr int kBwdFold = 4;    // chunks whose sums are held in FP32 pairs
 
 struct __align__(256) BwdWarp {
   unsigned char slot[kGroup][kSlotBytes];
@@ -298,8 +301,13 @@ struct PairSum {
     lo = __fadd2_rn(lo, __fadd2_rn(e, __fadd2_rn(d, f)));
     hi = t;
   }
-  __device__ __forceinline__ double total() const {
-    return ((double)hi.x + (double)hi.y) + ((double)lo.x + (double)lo.y);
+  __device__ __forceinline__ void clear() { hi = lo = make_float2(0.f, 0.f); }
+  // The sum of both, and back to zero; an infinite term leaves lo without meaning.
+  __device__ __forceinline__ double take() {
+    const float rest = (isfinite(hi.x) ? lo.x : 0.f) + (isfinite(hi.y) ? lo.y : 0.f);
+    const double s = (double)hi.x + (double)hi.y + (double)rest;
+    clear();
+    return s;
   }
 };
 
@@ -335,7 +343,10 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
   unsigned long long cblk = kEmpty;  // block the half's table belongs to
   uint32_t present = 0u;             // its digits that are in the map
   PairSum acc_f, acc_l;              // sum s G f, sum s G u^4 D d, by column
-  acc_f.hi = acc_f.lo = acc_l.hi = acc_l.lo = make_float2(0.f, 0.f);
+  acc_f.clear();
+  acc_l.clear();
+  double af = 0.0, al = 0.0;         // their sums over this lane's chunks
+  int chunks = 0;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + wid, nw = (int64_t)gridDim.x * kWarps;
   for (int64_t c = gw; c * kBwdChunk < a.p; c += nw) {
     const int64_t c1 = min(a.p, c * kBwdChunk + kBwdChunk);
@@ -470,8 +481,13 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
       }
       __syncwarp();  // the slots are rewritten by the next group
     }
+    if (++chunks % kBwdFold == 0) {  // warp-uniform
+      af += acc_f.take();
+      al += acc_l.take();
+    }
   }
-  double af = acc_f.total(), al = acc_l.total();
+  af += acc_f.take();
+  al += acc_l.take();
   for (int o = 16; o > 0; o >>= 1) {
     af += __shfl_down_sync(0xffffffffu, af, o);
     al += __shfl_down_sync(0xffffffffu, al, o);

@@ -234,3 +234,42 @@ def test_points_that_reach_no_voxel_add_nothing(sb, diff_case, lr):
     np.testing.assert_allclose(sc2, sc, rtol=2.0**-20)  # a point's sum by class is taken in FP32
     np.testing.assert_array_equal(gx2[~is_bad], gx)
     np.testing.assert_array_equal(gx2[is_bad], 0)
+
+
+def test_sums_over_a_set_leave_the_range_of_fp32(sb, diff_case):
+    """The sums over a training set are held beyond FP32's range.  G = 2^122 scales every FP32 operation of G = 1 by a
+    power of two, so the sums do as well (2^-38: the order of the FP64 additions), for a set whose terms add up past
+    3.4e38 many times over in every lane."""
+    c = diff_case
+    p = _params(sb, c["prm"])
+    xyzl = np.concatenate([c["xyz"], c["lab"][:, None].astype(np.float32)], 1)
+    big = np.tile(xyzl, (2000000 // len(xyzl) + 1, 1))
+    with sb.Map(p) as m:
+        m.insert_training(c["xyz"], c["lab"])
+        keys, alpha, _ = m.export()
+        got = []
+        for G in (1.0, 2.0**122):
+            m.grad_clear()
+            assert m.grad_add_alpha(keys, np.full(alpha.shape, G, np.float32)) == 0
+            got.append(m.backward(big, grad_xyz=False)[:2])
+    assert got[0][1] * 2.0**122 > 1e42
+    for one, scaled in zip(got[0], got[1]):
+        assert abs(scaled - one * 2.0**122) <= 2.0**-38 * abs(scaled)
+
+
+def test_an_infinite_upstream_gradient_gives_an_infinite_sum(sb):
+    """Points at voxel centres and l = 2.5 voxels: no pair's f is 0 by rounding (the nearest to l has d^2 = 6 res^2
+    against 6.25), so no term of the sum is 0 * inf."""
+    v = np.array([[0, 0, 0], [1, 0, 0], [4, 2, 1]])
+    xyz = ((v + 0.5) * 0.25).astype(np.float32)  # exact
+    lab = np.ones(len(v), np.int32)
+    p = sb.default_params(res=0.25, length_scale=0.625, num_classes=2, pool_blocks=1 << 10, sample_capacity=1 << 16)
+    with sb.Map(p) as m:
+        m.insert_training(xyz, lab)
+        m.grad_clear()
+        keys, alpha, _ = m.export()
+        G = np.ones(alpha.shape, np.float32)
+        G[(keys == [1, 0, 0]).all(1)] = np.inf
+        assert m.grad_add_alpha(keys, G) == 0
+        gs = m.backward(np.concatenate([xyz, lab[:, None].astype(np.float32)], 1), grad_xyz=False)[1]
+    assert gs == np.inf
