@@ -373,10 +373,27 @@ cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf
 cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems);
 // tiles.cu: the downsampling by occupied tiles.  The frame must fit the
 // scratch (tile_frame_fits), the items leave room for the flagged points
-// (tile_items_fit), and the occupied tiles not exceed tile_capacity.
+// (tile_items_fit), and the occupied tiles not exceed tile_limit.
 constexpr uint32_t kTilesDeclined = 1u << 30;  // an item outside the frame, or in a cell beyond 2^22
 constexpr int64_t kTileFrameMax = 1 << 22;  // directory entries per scan at most
 int64_t tile_capacity(int64_t sample_capacity);
+// Occupied tiles up to which the tile form takes an update: at most the room
+// (tile_capacity), and not so many that the sorted form is the faster one.  The
+// tile form's time grows by 2.5 us per 1000 tiles (4 KB of cells each, cleared,
+// counted and given offsets), 2.4 us per million directory entries and 7 per
+// million of one scan's frame; without them it is 32 us ahead, and 45 us more per
+// million items of neighbouring beams (beams in random order: nothing).  From 33
+// scans of 11k to 8.3M items, 680 to 199k tiles, and 8 batches, both forms
+// measured, in us sorted / tiles.  Ingest: 79k items in 2600 tiles 146 / 112;
+// 3.1M in 6300 351 / 221; 115k in 18k 152 / 161; 916k in 44k 205 / 314; 215k in
+// 55k, a frame of 3.9M entries 170 / 321.  Batches of 16: 1.1M items in 50k tiles
+// 401 / 534, 11M in 88k 1375 / 1111.  An update declined after marking pays about
+// 20 us for it, so the line lies 8000 tiles above `even`, where the forms are
+// equal, and where that is hardly above no tiles at all marking does not start (0).
+__host__ __device__ inline uint32_t tile_limit(uint32_t tile_cap, int64_t entries, int ns, int64_t items) {
+  const int64_t even = 12288 - entries / ns / 384 - entries / 1024 + items / 64;
+  return even < 2048 ? 0u : (even + 8192 < (int64_t)tile_cap ? (uint32_t)(even + 8192) : tile_cap);
+}
 bool tile_frame_fits(const MapState& m, int ns, const KeyFrame& kf);
 bool tile_items_fit(const MapState& m, int64_t nitems);
 // alone: the sorted form does not follow, an item outside the frame is an error; else it declines the tile form

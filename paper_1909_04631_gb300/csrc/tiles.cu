@@ -44,6 +44,10 @@ namespace {
 constexpr int kCells = 1 << kLocalBits;  // cells of a tile
 constexpr int kChunk = 256;              // directory entries per rank CTA, one per thread
 constexpr int kSuper = 256;              // chunks per second-level count
+// words from one second-level count to the next: a line each.  A sparse scan adds
+// up to its number of items to a few of them, and atomics on one line take turns
+// (side by side in two lines, marking 3.2M items of a 60 m scan took 91 us)
+constexpr int kSuperStep = 32;
 constexpr int kGroup = 256;              // tiles per count of training points
 constexpr uint32_t kBadPoint = 1u << 31;   // info word: the sums do not give the point's mean
 constexpr uint32_t kLowPoint = 1u << 30;   // info word: fractions of its members are in the list
@@ -62,7 +66,7 @@ struct LowPart {  // a member's fraction on one axis
 struct TileBufs {
   uint32_t* dir;       // [entries] 0, 1 marked, then rank + 1; chunk and second-level counts behind (keys)
   uint32_t* chunks;    // [entries / kChunk + 1] occupied tiles per chunk
-  uint32_t* supers;    // [chunks / kSuper + 1]
+  uint32_t* supers;    // [chunks / kSuper + 1] counts, kSuperStep words apart
   uint32_t* groups;    // [tile_cap / kGroup + 1] training points per kGroup tiles
   uint2* cells;        // [tile_cap * kCells] (label mask, first training point) (sitems)
   int4* tiles;         // [tile_cap] each occupied tile: index per axis, scan (seg_start)
@@ -183,7 +187,7 @@ struct Quotient {
 // Every item of the update through op.  A warp takes 32 consecutive points
 // (beams), a lane each, so the samples at the same place along neighbouring
 // beams, which mostly share a cell, meet in one warp: op.look sees the runs and
-// only their last lanes touch memory.  kPhases warps share 32 beams, each
+// only their last lanes touch memory; op.done ends the warp's share early.  kPhases warps share 32 beams, each
 // taking two samples of every 2 kPhases (two chains of dependent loads in
 // flight); the first also takes the hits.
 constexpr int kPhases = 8;
@@ -239,25 +243,45 @@ __device__ __forceinline__ void each_item(const TileArgs& a, Op& op) {
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) op.apply(found[u]);
+      if (op.done()) return;  // warp-uniform
     }
   }
 }
 
+__device__ __forceinline__ uint32_t limit_of(const TileArgs& a) {
+  return tile_limit(a.b.tile_cap, a.b.entries, a.ns, a.dc->n_items);
+}
 // whether the tile form takes this update (decided on the device; n_sort holds the answer
 // for the sorted form)
 __device__ __forceinline__ bool tiles_on(const TileArgs& a) {
-  return a.dc->err == 0 && a.dc->n_ttiles <= a.b.tile_cap && a.dc->n_items <= a.b.item_cap;
+  return a.dc->err == 0 && a.dc->n_ttiles <= limit_of(a) && a.dc->n_items <= a.b.item_cap;
 }
 __device__ __forceinline__ bool packed(const TileArgs& a) { return a.dc->max_points < a.pack_limit; }
 
 // ---------------------------------------------------------------- mark, rank
+// A warp adds its fresh tiles to the total in steps of kFlush and stops once the
+// total is past the limit: a sparse scan, whose items mostly have a tile each, is
+// declined after a small share of them.
+constexpr uint32_t kFlush = 16;
 struct MarkOp {
   struct Found {
     uint32_t entry, old;
   };
   const TileArgs& a;
+  uint32_t limit;
   uint32_t fresh = 0;
   bool out = false;
+  __device__ __forceinline__ bool done() {
+    const uint32_t w = __reduce_add_sync(0xffffffffu, fresh);
+    if (w < kFlush) return false;
+    uint32_t before = 0;
+    if ((threadIdx.x & 31) == 0) {
+      before = *(volatile const uint32_t*)&a.dc->n_ttiles;
+      if (before <= limit) before = atomicAdd(&a.dc->n_ttiles, w);
+    }
+    fresh = 0;
+    return __shfl_sync(0xffffffffu, before, 0) + w > limit;
+  }
   // A tile's word is mostly set already: a cached read first (it may be an old
   // 0), then one past the L1, so the tiles around the sensor do not serialise.
   __device__ __forceinline__ Found look(const Item& it, const Run& run) {
@@ -272,20 +296,36 @@ struct MarkOp {
   __device__ __forceinline__ void apply(const Found& f) {
     if (f.old == 0u && atomicExch(a.b.dir + f.entry, 1u) == 0u) {
       atomicAdd(a.b.chunks + f.entry / kChunk, 1u);
-      atomicAdd(a.b.supers + f.entry / (kChunk * kSuper), 1u);
+      atomicAdd(a.b.supers + f.entry / (kChunk * kSuper) * kSuperStep, 1u);
       ++fresh;
     }
   }
 };
+// The directory and its counts to zero, unless marking will not start.
+__global__ void __launch_bounds__(256) tile_clear_kernel(TileArgs a, uint32_t words) {
+  if (a.dc->err || a.dc->n_ttiles > limit_of(a)) return;  // neither changes in this launch
+  if (limit_of(a) == 0u) return;
+  uint4* const d = reinterpret_cast<uint4*>(a.b.dir);
+  const uint32_t i0 = blockIdx.x * 256 + threadIdx.x;
+  for (uint32_t i = i0; i < words / 4; i += gridDim.x * 256) d[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (i0 < (words & 3u)) a.b.dir[words / 4 * 4 + i0] = 0u;
+}
+
 __global__ void __launch_bounds__(256, 6) tile_mark_kernel(TileArgs a) {
-  // other CTAs of this launch may set the error or decline, so one read decides for the whole CTA: warps that
-  // went on without the others would miss each_item's scan offsets
+  // other CTAs of this launch may set the error, decline or pass the limit, so one read decides for the whole CTA:
+  // warps that went on without the others would miss each_item's scan offsets
   __shared__ int s_off;
-  if (threadIdx.x == 0)
-    s_off = *(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles >= kTilesDeclined;
+  const uint32_t limit = limit_of(a);
+  if (threadIdx.x == 0) {
+    s_off = *(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles > limit;
+    if (limit == 0u) {  // not even one tile
+      atomicMax(&a.dc->n_ttiles, kTilesDeclined);
+      s_off = 1;
+    }
+  }
   __syncthreads();
   if (s_off) return;
-  MarkOp op{a};
+  MarkOp op{a, limit};
   each_item(a, op);
   const uint32_t w = __reduce_add_sync(0xffffffffu, op.fresh);
   const bool out = __any_sync(0xffffffffu, op.out);
@@ -323,7 +363,7 @@ __global__ void __launch_bounds__(256) tile_rank_kernel(TileArgs a) {
     if (a.b.chunks[c] == 0u) continue;  // uniform over the CTA
     __syncthreads();
     uint32_t before = 0;
-    for (uint32_t k = threadIdx.x; k < c / kSuper; k += 256) before += a.b.supers[k];
+    for (uint32_t k = threadIdx.x; k < c / kSuper; k += 256) before += a.b.supers[k * kSuperStep];
     for (uint32_t k = c / kSuper * kSuper + threadIdx.x; k < c; k += 256) before += a.b.chunks[k];
     before = __reduce_add_sync(0xffffffffu, before);
     if (lane == 0) s_w[warp] = before;
@@ -371,6 +411,7 @@ struct MaskOp {
     }
     return f;
   }
+  __device__ __forceinline__ bool done() const { return false; }
   __device__ __forceinline__ void apply(const Found& f) {
     if ((f.old & f.bit) != f.bit) atomicOr(&a.b.cells[(size_t)f.rank * kCells + f.cell].x, f.bit);
   }
@@ -606,6 +647,7 @@ struct AddOp {
     f.bad = ((bads >> run.first) & (0xffffffffu >> (31 - at))) != 0u;
     return f;
   }
+  __device__ __forceinline__ bool done() const { return false; }
   __device__ __forceinline__ void apply(const Found& f) {
     if (f.p == kNoPoint) return;
     atomicAdd(a.b.sum[0] + f.p, f.d[0]);
@@ -729,6 +771,7 @@ struct GatherOp {
     }
     return f;
   }
+  __device__ __forceinline__ bool done() const { return false; }
   __device__ __forceinline__ void apply(const Found& f) {
     if (f.w != kNoPoint)
       a.b.gathered[atomicAdd(a.b.start + f.w, 1u)] = make_float4(f.x[0], f.x[1], f.x[2], 0.f);
@@ -765,7 +808,7 @@ TileArgs tile_args(const MapState& m, int ns, uint32_t entries, bool alone) {
   a.b.dir = reinterpret_cast<uint32_t*>(s.keys);
   a.b.chunks = a.b.dir + entries;
   a.b.supers = a.b.chunks + (entries / kChunk + 1);
-  a.b.groups = a.b.supers + ((entries / kChunk + 1) / kSuper + 1);
+  a.b.groups = a.b.supers + ((entries / kChunk + 1) / kSuper + 1) * kSuperStep;
   a.b.cells = reinterpret_cast<uint2*>(s.sitems);
   a.b.tile_cap = (uint32_t)tile_capacity(s.s_cap);
   a.b.tiles = reinterpret_cast<int4*>(s.seg_start);
@@ -801,7 +844,7 @@ TileArgs tile_args(const MapState& m, int ns, uint32_t entries, bool alone) {
 // Directory words of `entries` tiles, counts included.
 static int64_t directory_words(int64_t entries, int64_t tile_cap) {
   const int64_t chunks = entries / kChunk + 1;
-  return entries + chunks + (chunks / kSuper + 1) + (tile_cap / kGroup + 1);
+  return entries + chunks + (chunks / kSuper + 1) * kSuperStep + (tile_cap / kGroup + 1);
 }
 
 // Occupied tiles that the scratch of S items has room for (8 bytes a cell in 16 S bytes).
@@ -822,10 +865,11 @@ bool tile_items_fit(const MapState& m, int64_t nitems) {
 cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, bool alone) {
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
   const TileArgs a = tile_args(m, ns, entries, alone);
-  cudaError_t e = cudaMemsetAsync(a.b.dir, 0, sizeof(uint32_t) * (size_t)directory_words(entries, a.b.tile_cap), m.stream);
-  if (e != cudaSuccess) return e;
+  const int64_t words = directory_words(entries, a.b.tile_cap);
+  const unsigned blocks = (unsigned)std::min<int64_t>((words / 4 + 255) / 256 + 1, (int64_t)m.sm_count * 8);
+  tile_clear_kernel<<<blocks, 256, 0, m.stream>>>(a, (uint32_t)words);
   tile_mark_kernel<<<item_blocks(m, total_n), 256, 0, m.stream>>>(a);
-  m.launches += 1;
+  m.launches += 2;
   return cudaGetLastError();
 }
 
