@@ -220,3 +220,52 @@ def test_sparse_scans_take_the_sorted_form(sb, orc, kind, max_range, marked, til
     with sb.Map(sb.default_params(**prm, pool_blocks=1 << 18, sample_capacity=1 << 24, sensor_model=1)) as m:
         s = m.insert_batch([dict(points=pts, labels=lab, pose=T, map_id=0)] * 2)
         assert s["train_points"] == 2 * st["train"]
+
+
+def _crowd(n, at, rng):
+    """n hits within 3 cm of `at`: one cell of them, and one of their free samples at each place along the beams."""
+    return (np.asarray(at) + 0.03 * rng.random((n, 3))).astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["counts in their own word", "128-bit sums from a corner", "gathered"])
+def test_crowded_cells(sb, orc, kind):
+    """Branches that only a crowd of members reaches: more points than the counts that ride on the sums allow
+    (2^19 / 18 at this free-sample spacing), 2^15 members and more in cells off the corner of a tile at a coordinate
+    plane (both sides of it), and 2^18 of them, whose points are gathered."""
+    rng = np.random.default_rng(23)
+    step = 0.3
+    if kind == "counts in their own word":
+        pts, T, step = _crowd(30000, (0.3, 0.2, -0.15), rng), _pose(3.33, -2.2, 1.15), 0.01
+    elif kind == "128-bit sums from a corner":
+        pts, T = np.concatenate([_crowd(34000, (0.33, 0.53, 0.63), rng), _crowd(34000, (-0.37, -0.57, -0.27), rng)]), np.eye(4)
+    else:
+        pts, T = _crowd(270000, (0.33, 0.53, -0.27), rng), np.eye(4)
+    lab = np.ones(len(pts), np.int32)
+    prm = dict(res=0.1, length_scale=0.3, sigma0=0.4, alpha0=0.001, free_step=step, num_classes=2, max_range=50.0)
+    ox, ol, st = orc.training_set(orc.params(**prm), pts, lab, T)
+    with sb.Map(sb.default_params(**prm, pool_blocks=1 << 12, sample_capacity=1 << 22)) as m:
+        gx, gl = m.training_set(pts, lab, T)
+    o, g = np.lexsort((ol, *ox.T)), np.lexsort((gl, *gx.T))
+    np.testing.assert_array_equal(gl[g], ol[o])
+    np.testing.assert_array_equal(gx[g], ox[o])
+
+
+def test_a_batch_without_room_for_its_tiles(sb):
+    """Directories that fit and occupied tiles that do not (512 here): the recorded sorted form takes the batch, with
+    the map of single updates on a handle with room."""
+    rng = np.random.default_rng(29)
+    prm = dict(num_classes=3, max_range=15.0, pool_blocks=1 << 15, track_pairs=1)
+    scans = []
+    for i in range(3):
+        d = rng.normal(size=(150, 3))
+        pts = (d / np.linalg.norm(d, axis=1)[:, None] * rng.uniform(4, 14.5, (150, 1))).astype(np.float32)
+        scans.append(dict(points=pts, labels=rng.integers(1, 4, 150).astype(np.int32), pose=_pose(i, 0.3, -0.2, i), map_id=0))
+    with sb.Map(sb.default_params(**prm, sample_capacity=1 << 17)) as mb, \
+            sb.Map(sb.default_params(**prm, sample_capacity=1 << 22)) as ms:
+        st = mb.insert_batch(scans)
+        train = sum(ms.insert_scan(s["points"], s["labels"], s["pose"])["train_points"] for s in scans)
+        (kb, ab, pb), (ks, as_, ps) = mb.export(pairs=True), ms.export(pairs=True)
+    assert st["train_points"] == train
+    np.testing.assert_array_equal(kb, ks)
+    np.testing.assert_array_equal(pb, ps)
+    np.testing.assert_allclose(ab, as_, rtol=1e-5)  # sums in another order
