@@ -143,15 +143,23 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
   __shared__ int64_t s_off[kMaxScans + 1];
   __shared__ int s_box[6];
   __shared__ unsigned long long s_total;
+  __shared__ uint32_t s_longest;
   for (int t = threadIdx.x; t <= ns; t += blockDim.x) s_off[t] = desc[t].off;
   if (threadIdx.x < 6) s_box[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : INT_MIN;
-  if (threadIdx.x == 6) s_total = 0ull;
+  if (threadIdx.x == 6) {
+    s_total = 0ull;
+    s_longest = 0u;
+  }
   __syncthreads();
   const int64_t total = s_off[ns];
   int tlo[3] = {INT_MAX, INT_MAX, INT_MAX}, thi[3] = {INT_MIN, INT_MIN, INT_MIN};
   unsigned long long sum = 0ull;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    sum += transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tlo, thi);
+  uint32_t longest = 0u;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long c = transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tlo, thi);
+    sum += c;
+    longest = max(longest, (uint32_t)(c & kFreeMask));
+  }
   // tile bounding box of the kept hits: warp, then CTA, then one global atomic per CTA and bound
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -163,12 +171,17 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&s_total, sum);
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if ((threadIdx.x & 31) == 0 && sum) {
+    atomicAdd(&s_total, sum);
+    atomicMax(&s_longest, longest);
+  }
   __syncthreads();
   if (threadIdx.x < 3 && s_box[threadIdx.x] <= s_box[3 + threadIdx.x]) {
     atomicMin(&dc->tbox[threadIdx.x], s_box[threadIdx.x]);
     atomicMax(&dc->tbox[3 + threadIdx.x], s_box[3 + threadIdx.x]);
   }
+  if (threadIdx.x == 32 && s_longest) atomicMax(&dc->longest, s_longest);  // read by later launches
   if (threadIdx.x == 0) {  // the last CTA to finish (a counter after a fence) has the total
     atomicAdd(&dc->n_total, s_total);
     __threadfence();

@@ -128,6 +128,7 @@ __global__ void begin_kernel(DevCounters* dc, uint32_t epoch, uint32_t n_points)
   dc->n_scan = 0;
   dc->n_total = 0;
   dc->n_ttiles = 0;
+  dc->longest = 0;
   dc->n_wide = 0;
   dc->n_low = 0;
   dc->n_gather = 0;
@@ -159,6 +160,7 @@ __global__ void batch_begin_kernel(DevCounters* dc, const ScanDesc* desc, int ns
   dc->n_scan = 0;
   dc->n_total = 0;
   dc->n_ttiles = 0;
+  dc->longest = 0;
   dc->n_wide = 0;
   dc->n_low = 0;
   dc->n_gather = 0;
@@ -481,11 +483,7 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   // max_range fits a directory, the tiles are marked before the counters come
   // back, so the read-back also tells how many are occupied (or that items lie
   // outside: a pose that scales or shears; the fitted frame below holds them).
-  const uint32_t tile_cap = (uint32_t)tile_capacity(m.s.s_cap);
-  const int64_t entries = (int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2];
-  // even the most items that a rigid pose can give would be too few for a directory of this size: not marked
-  const double most_items = std::min((double)n * (1.0 + m.prm.max_range / m.prm.free_step), 1e12);
-  const bool marked = !probs && tile_frame_fits(m, 1, kf) && tile_limit(tile_cap, entries, 1, (int64_t)most_items) > 0;
+  const bool marked = !probs && tile_frame_fits(m, 1, kf);
   if (marked) CK(&m, launch_tile_mark(m, 1, n, kf, false));
   if (probs) CK(&m, launch_offsets(m, n));  // the sorted form for certain: while the host waits
   st = read_counters(m);
@@ -493,7 +491,7 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   if (m.hc->err != 0) return status_from_device(m);
   *nitems = m.hc->n_items;
   if (*nitems == 0) return SBKI_OK;
-  if (marked && m.hc->n_ttiles <= tile_limit(tile_cap, entries, 1, *nitems) && tile_items_fit(m, *nitems)) {
+  if (marked && tile_gate(m, 1, kf).takes(*m.hc)) {
     CK(&m, launch_tiles(m, 1, n, kf, *nitems));
     return SBKI_OK;
   }
@@ -510,12 +508,15 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   }
   CK(&m, cudaMemcpyAsync(m.s.desc, &fitted, sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
   // a frame fitted to the hits that cannot hold more tiles than the limit
-  const int64_t fitted_entries = (int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2];
-  if (!probs && !marked && m.hc->n_ttiles < kTilesDeclined && tile_frame_fits(m, 1, kf) && tile_items_fit(m, *nitems) &&
-      std::min<int64_t>(fitted_entries, *nitems) <= tile_limit(tile_cap, fitted_entries, 1, *nitems)) {
-    CK(&m, launch_tile_mark(m, 1, n, kf, true));
-    CK(&m, launch_tiles(m, 1, n, kf, *nitems));
-    return SBKI_OK;
+  if (!probs && !marked && m.hc->n_ttiles < kTilesDeclined && tile_frame_fits(m, 1, kf)) {
+    const TileGate gate = tile_gate(m, 1, kf);
+    DevCounters most = *m.hc;
+    most.n_ttiles = std::min(gate.entries, most.n_items);
+    if (gate.takes(most)) {
+      CK(&m, launch_tile_mark(m, 1, n, kf, true));
+      CK(&m, launch_tiles(m, 1, n, kf, *nitems));
+      return SBKI_OK;
+    }
   }
   if (!probs) CK(&m, launch_offsets(m, n));
   CK(&m, launch_emit(m, 1, n, kf, probs ? m.s.hit_src : nullptr));

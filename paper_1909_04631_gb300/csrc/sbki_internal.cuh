@@ -61,6 +61,7 @@ struct DevCounters {
   uint32_t n_wide;                    // tile form: training points left to the gathered exact mean
   uint32_t n_gather;                  // tile form: their members
   uint32_t max_points;                // points of the update's largest scan
+  uint32_t longest;                   // free samples of the longest beam
 };
 
 // per-point sample counts of a1/a2: kept hits in bits 40.., free samples below
@@ -373,29 +374,45 @@ cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf
 cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems);
 // tiles.cu: the downsampling by occupied tiles.  The frame must fit the
 // scratch (tile_frame_fits), the items leave room for the flagged points
-// (tile_items_fit), and the occupied tiles not exceed tile_limit.
+// (item_cap), and the occupied tiles not exceed TileGate::limit.
 constexpr uint32_t kTilesDeclined = 1u << 30;  // an item outside the frame, or in a cell beyond 2^22
 constexpr int64_t kTileFrameMax = 1 << 22;  // directory entries per scan at most
 int64_t tile_capacity(int64_t sample_capacity);
-// Occupied tiles up to which the tile form takes an update: at most the room
-// (tile_capacity), and not so many that the sorted form is the faster one.  The
-// tile form's time grows by 2.5 us per 1000 tiles (4 KB of cells each, cleared,
-// counted and given offsets), 2.4 us per million directory entries and 7 per
-// million of one scan's frame; without them it is 32 us ahead, and 45 us more per
-// million items of neighbouring beams (beams in random order: nothing).  From 33
-// scans of 11k to 8.3M items, 680 to 199k tiles, and 8 batches, both forms
-// measured, in us sorted / tiles.  Ingest: 79k items in 2600 tiles 146 / 112;
-// 3.1M in 6300 351 / 221; 115k in 18k 152 / 161; 916k in 44k 205 / 314; 215k in
-// 55k, a frame of 3.9M entries 170 / 321.  Batches of 16: 1.1M items in 50k tiles
-// 401 / 534, 11M in 88k 1375 / 1111.  An update declined after marking pays about
-// 20 us for it, so the line lies 8000 tiles above `even`, where the forms are
-// equal, and where that is hardly above no tiles at all marking does not start (0).
-__host__ __device__ inline uint32_t tile_limit(uint32_t tile_cap, int64_t entries, int ns, int64_t items) {
-  const int64_t even = 12288 - entries / ns / 384 - entries / 1024 + items / 64;
-  return even < 2048 ? 0u : (even + 8192 < (int64_t)tile_cap ? (uint32_t)(even + 8192) : tile_cap);
-}
+// Whether an update whose tiles were marked is the tile form's, on the host and
+// on the device (one decision: integers only).
+//
+// limit: the occupied tiles up to which it is.  At most the room (tile_cap), and
+// not so many that the sorted form is the faster one.  Against the sorted form the
+// tile form gains, in tiles of 2.55 us per 1000 (4 KB of cells each, cleared,
+// counted and given offsets): 0 to 39 us by the items (few items sort quickly) and
+// 45 us per million items of neighbouring beams (beams in random order: nothing);
+// it loses 0.25 us per sample of the longest beam above 50 (three passes walk
+// along it) and 2.4 us per million directory entries.  From 63 scans of 34 to 8.3M
+// items, up to 199k tiles and 200 samples a beam, and 8 batches, both forms
+// measured, in us sorted / tiles.  Ingest: 165 items of one 50 m beam 92 / 119; 12k
+// of 500 such beams 134 / 138; 8400 of 500 beams of 15 m 133 / 100; 79k items in
+// 2600 tiles 146 / 112; 3.1M in 6300 351 / 221; 916k in 44k 205 / 314; 215k in 55k
+// 170 / 321.  Batches of 16: 1.1M items in 50k tiles 401 / 534, 11M in 88k 1375 /
+// 1111.  An update declined after marking pays about 20 us for it, so the line lies
+// 8000 tiles above `even`, where the forms are equal; where that is no tile at all
+// marking does not start (0), which leaves two idle launches, about 7 us.
+struct TileGate {
+  uint32_t tile_cap, item_cap;
+  uint32_t entries;  // of the directory
+  __host__ __device__ uint32_t limit(uint32_t items, uint32_t longest) const {
+    const uint32_t few = items < 65536u ? items : 65536u;
+    const int32_t gain = (int32_t)(15360u * few / (few + 2304u) + items / 64u);  // items <= 2^27
+    const int32_t loss = 98 * ((longest < 200000u ? (int32_t)longest : 200000) - 50) + (int32_t)(entries / 1024u);
+    const int32_t even = longest > 50u ? gain - loss : gain - (int32_t)(entries / 1024u);
+    return even <= 0 ? 0u : ((uint32_t)even + 8192u < tile_cap ? (uint32_t)even + 8192u : tile_cap);
+  }
+  __host__ __device__ uint32_t limit(const DevCounters& c) const { return limit(c.n_items, c.longest); }
+  __host__ __device__ bool takes(const DevCounters& c) const {
+    return c.err == 0 && c.n_ttiles <= limit(c) && c.n_items <= item_cap;
+  }
+};
 bool tile_frame_fits(const MapState& m, int ns, const KeyFrame& kf);
-bool tile_items_fit(const MapState& m, int64_t nitems);
+TileGate tile_gate(const MapState& m, int ns, const KeyFrame& kf);  // of a frame that fits
 // alone: the sorted form does not follow, an item outside the frame is an error; else it declines the tile form
 cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, bool alone);
 cudaError_t launch_tiles(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, int64_t nitems);

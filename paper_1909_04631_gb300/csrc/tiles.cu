@@ -81,7 +81,6 @@ struct TileBufs {
   float4* gathered;    // [members of flagged points] (items, when the sums are done)
   uint32_t entries;
   uint32_t tile_cap;
-  uint32_t item_cap;   // items that leave room for as many flagged points
 };
 
 struct TileArgs {
@@ -94,6 +93,7 @@ struct TileArgs {
   float4* train;
   DevCounters* dc;
   bool alone;           // no sorted form behind: an item outside the frame is an error
+  TileGate gate;
   uint32_t pack_limit;  // scans of fewer points have no cell of 2^19 members: counts ride on the sums
 };
 
@@ -248,14 +248,9 @@ __device__ __forceinline__ void each_item(const TileArgs& a, Op& op) {
   }
 }
 
-__device__ __forceinline__ uint32_t limit_of(const TileArgs& a) {
-  return tile_limit(a.b.tile_cap, a.b.entries, a.ns, a.dc->n_items);
-}
 // whether the tile form takes this update (decided on the device; n_sort holds the answer
 // for the sorted form)
-__device__ __forceinline__ bool tiles_on(const TileArgs& a) {
-  return a.dc->err == 0 && a.dc->n_ttiles <= limit_of(a) && a.dc->n_items <= a.b.item_cap;
-}
+__device__ __forceinline__ bool tiles_on(const TileArgs& a) { return a.gate.takes(*a.dc); }
 __device__ __forceinline__ bool packed(const TileArgs& a) { return a.dc->max_points < a.pack_limit; }
 
 // ---------------------------------------------------------------- mark, rank
@@ -303,8 +298,8 @@ struct MarkOp {
 };
 // The directory and its counts to zero, unless marking will not start.
 __global__ void __launch_bounds__(256) tile_clear_kernel(TileArgs a, uint32_t words) {
-  if (a.dc->err || a.dc->n_ttiles > limit_of(a)) return;  // neither changes in this launch
-  if (limit_of(a) == 0u) return;
+  if (a.dc->err || a.dc->n_ttiles > a.gate.limit(*a.dc)) return;  // neither changes in this launch
+  if (a.gate.limit(*a.dc) == 0u) return;
   uint4* const d = reinterpret_cast<uint4*>(a.b.dir);
   const uint32_t i0 = blockIdx.x * 256 + threadIdx.x;
   for (uint32_t i = i0; i < words / 4; i += gridDim.x * 256) d[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -315,7 +310,7 @@ __global__ void __launch_bounds__(256, 6) tile_mark_kernel(TileArgs a) {
   // other CTAs of this launch may set the error, decline or pass the limit, so one read decides for the whole CTA:
   // warps that went on without the others would miss each_item's scan offsets
   __shared__ int s_off;
-  const uint32_t limit = limit_of(a);
+  const uint32_t limit = a.gate.limit(*a.dc);
   if (threadIdx.x == 0) {
     s_off = *(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles > limit;
     if (limit == 0u) {  // not even one tile
@@ -801,7 +796,7 @@ unsigned item_blocks(const MapState& m, int64_t total_n) {
       1, std::min<int64_t>(((total_n + 31) / 32 * kPhases + 7) / 8, (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm));
 }
 
-TileArgs tile_args(const MapState& m, int ns, uint32_t entries, bool alone) {
+TileArgs tile_args(const MapState& m, int ns, uint32_t entries, const KeyFrame& kf, bool alone) {
   const Scratch& s = m.s;
   TileArgs a;
   a.g = m.g;
@@ -831,7 +826,7 @@ TileArgs tile_args(const MapState& m, int ns, uint32_t entries, bool alone) {
   a.train = s.train;
   a.dc = m.dc;
   a.alone = alone;
-  a.b.item_cap = (uint32_t)std::max<int64_t>(0, s.s_cap - 5 * (int64_t)a.b.tile_cap - 1);
+  a.gate = tile_gate(m, ns, kf);
   // a beam's samples lie `step` apart, so at most 1 + sqrt(3) ds / step of them are in one cell
   // (widened for FP32 positions); a point's members are hits (one a beam) or samples, never both
   const double per_beam = 1.0 + std::floor(1.74 * (double)m.g.ds / (double)m.g.step);
@@ -857,14 +852,19 @@ bool tile_frame_fits(const MapState& m, int ns, const KeyFrame& kf) {
   return e > 0 && e <= kTileFrameMax && directory_words(e * ns, tile_capacity(m.s.s_cap)) <= 2 * m.s.s_cap && tile_capacity(m.s.s_cap) > 0;
 }
 
-bool tile_items_fit(const MapState& m, int64_t nitems) {
+TileGate tile_gate(const MapState& m, int ns, const KeyFrame& kf) {
+  const int64_t cap = tile_capacity(m.s.s_cap);
+  TileGate t;
+  t.tile_cap = (uint32_t)cap;
   // as many flagged points as items find room in seg_start, behind the tiles
-  return nitems + 5 * tile_capacity(m.s.s_cap) + 1 <= m.s.s_cap;
+  t.item_cap = (uint32_t)std::max<int64_t>(0, m.s.s_cap - 5 * cap - 1);
+  t.entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
+  return t;
 }
 
 cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, bool alone) {
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
-  const TileArgs a = tile_args(m, ns, entries, alone);
+  const TileArgs a = tile_args(m, ns, entries, kf, alone);
   const int64_t words = directory_words(entries, a.b.tile_cap);
   const unsigned blocks = (unsigned)std::min<int64_t>((words / 4 + 255) / 256 + 1, (int64_t)m.sm_count * 8);
   tile_clear_kernel<<<blocks, 256, 0, m.stream>>>(a, (uint32_t)words);
@@ -875,7 +875,7 @@ cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFram
 
 cudaError_t launch_tiles(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, int64_t nitems) {
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
-  const TileArgs a = tile_args(m, ns, entries, false);
+  const TileArgs a = tile_args(m, ns, entries, kf, false);
   const unsigned blocks = item_blocks(m, total_n);
   const int64_t sms = m.sm_count;
   tile_rank_kernel<<<(unsigned)std::min<int64_t>(entries / kChunk + 1, 8 * sms), 256, 0, m.stream>>>(a);

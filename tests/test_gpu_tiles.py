@@ -186,8 +186,8 @@ def test_batch_with_items_past_the_frame_but_within_the_keys(sb):
 
 
 def _beams(kind, rng):
-    """Directions and ranges: lone beams all over a 60 m or 30 m scene, or a dense fan of beams close by."""
-    n, r1 = {"lone60": (200, 59), "lone30": (4000, 29), "fan": (4000, 12)}[kind]
+    """Directions and ranges: lone beams all over a 60 m or 30 m scene, a dense fan of beams close by, or five."""
+    n, r1 = {"lone60": (200, 59), "lone30": (4000, 29), "fan": (4000, 12), "few": (5, 49)}[kind]
     az, el = rng.uniform(0, 2 * np.pi, n), rng.uniform(-0.3, 0.3, n)
     if kind == "fan":
         az = np.linspace(0, 0.4, n)
@@ -195,11 +195,11 @@ def _beams(kind, rng):
     return np.stack([r * np.cos(el) * np.cos(az), r * np.cos(el) * np.sin(az), r * np.sin(el)], 1).astype(np.float32)
 
 
-@pytest.mark.parametrize("kind,max_range,marked,tiles", [("fan", 50.0, True, True), ("lone60", 60.0, False, False),
-                                                         ("lone30", 30.0, True, False)])
-def test_sparse_scans_take_the_sorted_form(sb, orc, kind, max_range, marked, tiles):
-    """Scans with hardly more items than occupied tiles: declined before or while their tiles are marked, and the
-    oracle's training set either way, alone and in a batch."""
+@pytest.mark.parametrize("kind,max_range,tiles", [("fan", 50.0, True), ("lone60", 60.0, False), ("lone30", 30.0, False),
+                                                  ("few", 50.0, False)])
+def test_sparse_scans_take_the_sorted_form(sb, orc, kind, max_range, tiles):
+    """Scans with hardly more items than occupied tiles, or a few long beams: declined before or while their tiles are
+    marked, and the oracle's training set either way, alone and in a batch."""
     rng = np.random.default_rng(17)
     pts = _beams(kind, rng)
     lab = rng.integers(1, 4, len(pts)).astype(np.int32)
@@ -213,10 +213,10 @@ def test_sparse_scans_take_the_sorted_form(sb, orc, kind, max_range, marked, til
     o, g = np.lexsort((ol, *ox.T)), np.lexsort((gl, *gx.T))
     np.testing.assert_array_equal(gl[g], ol[o])
     np.testing.assert_array_equal(gx[g], ox[o])
-    # begin, transform, then clear, mark and eight more; or offsets, emit, digit counts, a pass per byte of the key, three
+    # begin, transform, clear, mark, then eight more; or offsets, emit, digit counts, a pass per byte of the key, three
     tile = np.floor(np.concatenate([pts @ T[:3, :3].T + T[:3, 3], T[None, :3, 3]]) / 0.1).astype(int) >> 3
     bits = sum(int(np.ceil(np.log2(e))) for e in tile.max(0) - tile.min(0) + 3) + 9 + 2
-    assert launches == (12 if tiles else (4 if marked else 2) + 3 + -(-bits // 8) + 3)
+    assert launches == (12 if tiles else 4 + 3 + -(-bits // 8) + 3)
     with sb.Map(sb.default_params(**prm, pool_blocks=1 << 18, sample_capacity=1 << 24, sensor_model=1)) as m:
         s = m.insert_batch([dict(points=pts, labels=lab, pose=T, map_id=0)] * 2)
         assert s["train_points"] == 2 * st["train"]
