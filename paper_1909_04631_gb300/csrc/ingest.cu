@@ -55,7 +55,7 @@ __device__ __forceinline__ int map_of_segment(unsigned long long key, const KeyF
 // a1 for global point i of scan d
 __device__ __forceinline__ unsigned long long transform_count_one(const ScanDesc& d, int64_t i, const int64_t* off, const Geom& g,
                                                     float4* __restrict__ world, unsigned long long* __restrict__ cnt,
-                                                    DevCounters* dc, int tlo[3], int thi[3]) {
+                                                    DevCounters* dc, int tile[3], int tlo[3], int thi[3]) {
   const int64_t li = i - d.off;
   const float px = d.pts[3 * li], py = d.pts[3 * li + 1], pz = d.pts[3 * li + 2];
   int lab;
@@ -106,7 +106,7 @@ __device__ __forceinline__ unsigned long long transform_count_one(const ScanDesc
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const float q = __fmul_rn(wc[a], g.inv_ds);
-        const int t = floor_i(q) >> kTileShift;
+        const int t = tile[a] = floor_i(q) >> kTileShift;
         if (!(fabsf(q) < 4194304.0f)) atomicMax(&dc->n_ttiles, kTilesDeclined);  // no rigid pose reaches that far
         tlo[a] = min(tlo[a], t);
         thi[a] = max(thi[a], t);
@@ -143,22 +143,29 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
   __shared__ int64_t s_off[kMaxScans + 1];
   __shared__ int s_box[6];
   __shared__ unsigned long long s_total;
-  __shared__ uint32_t s_longest;
+  __shared__ uint32_t s_longest, s_near;
   for (int t = threadIdx.x; t <= ns; t += blockDim.x) s_off[t] = desc[t].off;
   if (threadIdx.x < 6) s_box[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : INT_MIN;
   if (threadIdx.x == 6) {
     s_total = 0ull;
-    s_longest = 0u;
+    s_longest = s_near = 0u;
   }
   __syncthreads();
   const int64_t total = s_off[ns];
   int tlo[3] = {INT_MAX, INT_MAX, INT_MAX}, thi[3] = {INT_MIN, INT_MIN, INT_MIN};
   unsigned long long sum = 0ull;
-  uint32_t longest = 0u;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long c = transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tlo, thi);
+  uint32_t longest = 0u, near = 0u;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < total; i0 += (int64_t)gridDim.x * blockDim.x) {  // CTA-uniform
+    const int64_t i = i0 + threadIdx.x;
+    unsigned long long c = 0ull;
+    int tile[3] = {INT_MIN / 2, 0, 0};  // of a kept hit
+    if (i < total) c = transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tile, tlo, thi);
     sum += c;
     longest = max(longest, (uint32_t)(c & kFreeMask));
+    int apart = 0;  // tiles to the next point's hit
+#pragma unroll
+    for (int a = 0; a < 3; ++a) apart = max(apart, abs(tile[a] - __shfl_down_sync(0xffffffffu, tile[a], 1)));
+    near += apart <= 1 && c != 0ull && (threadIdx.x & 31) != 31 ? 1u : 0u;
   }
   // tile bounding box of the kept hits: warp, then CTA, then one global atomic per CTA and bound
 #pragma unroll
@@ -172,16 +179,21 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
   longest = __reduce_max_sync(0xffffffffu, longest);
+  near = __reduce_add_sync(0xffffffffu, near);
   if ((threadIdx.x & 31) == 0 && sum) {
     atomicAdd(&s_total, sum);
     atomicMax(&s_longest, longest);
+    atomicAdd(&s_near, near);
   }
   __syncthreads();
   if (threadIdx.x < 3 && s_box[threadIdx.x] <= s_box[3 + threadIdx.x]) {
     atomicMin(&dc->tbox[threadIdx.x], s_box[threadIdx.x]);
     atomicMax(&dc->tbox[3 + threadIdx.x], s_box[3 + threadIdx.x]);
   }
-  if (threadIdx.x == 32 && s_longest) atomicMax(&dc->longest, s_longest);  // read by later launches
+  if (threadIdx.x == 32 && s_total) {  // read by later launches
+    atomicMax(&dc->longest, s_longest);
+    atomicAdd(&dc->n_near, s_near);
+  }
   if (threadIdx.x == 0) {  // the last CTA to finish (a counter after a fence) has the total
     atomicAdd(&dc->n_total, s_total);
     __threadfence();

@@ -129,6 +129,7 @@ __global__ void begin_kernel(DevCounters* dc, uint32_t epoch, uint32_t n_points)
   dc->n_total = 0;
   dc->n_ttiles = 0;
   dc->longest = 0;
+  dc->n_near = 0;
   dc->n_wide = 0;
   dc->n_low = 0;
   dc->n_gather = 0;
@@ -161,6 +162,7 @@ __global__ void batch_begin_kernel(DevCounters* dc, const ScanDesc* desc, int ns
   dc->n_total = 0;
   dc->n_ttiles = 0;
   dc->longest = 0;
+  dc->n_near = 0;
   dc->n_wide = 0;
   dc->n_low = 0;
   dc->n_gather = 0;

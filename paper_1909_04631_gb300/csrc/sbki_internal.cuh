@@ -62,6 +62,7 @@ struct DevCounters {
   uint32_t n_gather;                  // tile form: their members
   uint32_t max_points;                // points of the update's largest scan
   uint32_t longest;                   // free samples of the longest beam
+  uint32_t n_near;                    // kept hits within a tile of the next point's (31 of every 32 points counted)
 };
 
 // per-point sample counts of a1/a2: kept hits in bits 40.., free samples below
@@ -385,28 +386,30 @@ int64_t tile_capacity(int64_t sample_capacity);
 // not so many that the sorted form is the faster one.  Against the sorted form the
 // tile form gains, in tiles of 2.55 us per 1000 (4 KB of cells each, cleared,
 // counted and given offsets): 0 to 39 us by the items (few items sort quickly) and
-// 45 us per million items of neighbouring beams (beams in random order: nothing);
-// it loses 0.25 us per sample of the longest beam above 50 (three passes walk
-// along it) and 2.4 us per million directory entries.  From 63 scans of 34 to 8.3M
-// items, up to 199k tiles and 200 samples a beam, and 8 batches, both forms
-// measured, in us sorted / tiles.  Ingest: 165 items of one 50 m beam 92 / 119; 12k
-// of 500 such beams 134 / 138; 8400 of 500 beams of 15 m 133 / 100; 79k items in
-// 2600 tiles 146 / 112; 3.1M in 6300 351 / 221; 916k in 44k 205 / 314; 215k in 55k
-// 170 / 321.  Batches of 16: 1.1M items in 50k tiles 401 / 534, 11M in 88k 1375 /
-// 1111.  An update declined after marking pays about 20 us for it, so the line lies
-// 8000 tiles above `even`, where the forms are equal; where that is no tile at all
-// marking does not start (0), which leaves two idle launches, about 7 us.
+// 45 us per million items of beams that lie beside the next ones (others: nothing;
+// n_near tells); it loses 0.25 us per sample of the longest beam above 50 (three
+// passes walk along it) and 2.4 us per million directory entries.  From 63 scans
+// of 34 to 8.3M items, up to 199k tiles and 200 samples a beam, and 8 batches, both
+// forms measured, in us sorted / tiles.  Ingest: 165 items of one 50 m beam 92 /
+// 119; 12k of 500 such beams 134 / 138; 8400 of 500 beams of 15 m 133 / 100; 79k
+// items in 2600 tiles 146 / 112; 3.1M in 6300 351 / 221; 916k in 44k, beams in
+// random order, 205 / 314; 215k in 55k 170 / 321.  Batches of 16: 1.1M items in 50k
+// tiles 401 / 534, 11M in 88k 1375 / 1111.  An update declined after marking pays
+// 20 to 50 us for it, so the line lies 8000 tiles above `even`, where the forms are
+// equal (at `even`, shuffled street scans took 263 and 425 us for 249 and 379);
+// where that is no tile at all marking does not start (0), which leaves two idle
+// launches, about 7 us.
 struct TileGate {
   uint32_t tile_cap, item_cap;
   uint32_t entries;  // of the directory
-  __host__ __device__ uint32_t limit(uint32_t items, uint32_t longest) const {
-    const uint32_t few = items < 65536u ? items : 65536u;
-    const int32_t gain = (int32_t)(15360u * few / (few + 2304u) + items / 64u);  // items <= 2^27
-    const int32_t loss = 98 * ((longest < 200000u ? (int32_t)longest : 200000) - 50) + (int32_t)(entries / 1024u);
-    const int32_t even = longest > 50u ? gain - loss : gain - (int32_t)(entries / 1024u);
+  __host__ __device__ uint32_t limit(const DevCounters& c) const {  // 32 bits hold all of it: n_items <= 2^27
+    const uint32_t few = c.n_items < 65536u ? c.n_items : 65536u;
+    const uint32_t beside = c.n_valid ? 32u * c.n_near / c.n_valid : 0u;  // of 32
+    const uint32_t gain = 15360u * few / (few + 2304u) + c.n_items / 64u * beside / 32u;
+    const uint32_t longest = c.longest < 50u ? 0u : (c.longest < 200000u ? c.longest - 50u : 200000u);
+    const int32_t even = (int32_t)gain - (int32_t)(98u * longest + entries / 1024u);
     return even <= 0 ? 0u : ((uint32_t)even + 8192u < tile_cap ? (uint32_t)even + 8192u : tile_cap);
   }
-  __host__ __device__ uint32_t limit(const DevCounters& c) const { return limit(c.n_items, c.longest); }
   __host__ __device__ bool takes(const DevCounters& c) const {
     return c.err == 0 && c.n_ttiles <= limit(c) && c.n_items <= item_cap;
   }

@@ -269,3 +269,28 @@ def test_a_batch_without_room_for_its_tiles(sb):
     np.testing.assert_array_equal(kb, ks)
     np.testing.assert_array_equal(pb, ps)
     np.testing.assert_allclose(ab, as_, rtol=1e-5)  # sums in another order
+
+
+@pytest.mark.parametrize("order", ["along the rings", "shuffled"])
+def test_beams_without_neighbours_decline_sooner(sb, orc, order):
+    """A scan wide for its items: ordered beams (whose items meet in runs) take the tile form, the same beams shuffled
+    the sorted one; the same bits."""
+    rng = np.random.default_rng(31)
+    az, el = np.meshgrid(np.arange(1500) * (2 * np.pi / 1500), np.deg2rad(np.linspace(-24, -4, 20)))
+    r = np.minimum(1.73 / np.sin(-el.ravel()), 22.0)
+    az, el = az.ravel(), el.ravel()
+    pts = np.stack([r * np.cos(el) * np.cos(az), r * np.cos(el) * np.sin(az), r * np.sin(el)], 1).astype(np.float32)
+    if order == "shuffled":
+        pts = pts[rng.permutation(len(pts))]
+    lab = np.ones(len(pts), np.int32)
+    T = _pose(0.3, -1.75, 1.73)
+    prm = dict(res=0.1, length_scale=0.3, sigma0=0.4, alpha0=0.001, free_step=0.1, num_classes=3, max_range=60.0)
+    ox, ol, st = orc.training_set(orc.params(**prm), pts, lab, T)
+    with sb.Map(sb.default_params(**prm, pool_blocks=1 << 12, sample_capacity=1 << 24)) as m:
+        before = m.profile_read()["launches"]
+        gx, gl = m.training_set(pts, lab, T)
+        launches = m.profile_read()["launches"] - before
+    assert (launches == 12) == (order != "shuffled")
+    o, g = np.lexsort((ol, *ox.T)), np.lexsort((gl, *gx.T))
+    np.testing.assert_array_equal(gl[g], ol[o])
+    np.testing.assert_array_equal(gx[g], ox[o])
