@@ -94,9 +94,11 @@ typedef struct sbki_params {
                         * f(d/l_k) with support d < l_k = length_scale * l_scale[k] (Sec. V and VI
                         * name class-dependent parameters; reading K16).  Entries 0..K finite and
                         * > 0, l_k <= 0.75 * block_edge * res; sbki_default_params sets 1 (the
-                        * common l).  With any entry other than 1 the update takes the general
-                        * weighted accumulation; the block-major form, extended-block association
-                        * and the differentiable entry points refuse it */
+                        * common l).  With any entry other than 1, classes with l_k above about 3.5
+                        * voxels (and all classes, where one has l_k below half the voxel diagonal)
+                        * take the general weighted accumulation, slower than the common one; the
+                        * block-major form, extended-block association and the differentiable entry
+                        * points refuse it */
 } sbki_params;
 
 /* Per-insert counters (all for the last insert). */
@@ -228,10 +230,12 @@ typedef struct sbki_scan {
 sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t count, sbki_stats* stats);
 
 /* Launch shapes of the update's kernels (all persistent grids): CTAs per SM
- * for the accumulation (0 = as many as fit), training points per warp chunk
- * in the accumulation (1..64), CTAs per SM for the touched-block pass and for
- * the ingest kernels (transform, samples, segments, centroids).  Results do
- * not depend on them; speed does.  sbki_set_tuning drops the recorded
+ * for the accumulation (0 = as many as fit), the most training points a warp
+ * of the accumulation takes at once, in pairs (1..64; rounded up to whole
+ * groups of eight points, fewer where few points would leave less than three
+ * chunks per warp, at most 16 points for soft labels), CTAs per SM for the
+ * touched-block pass and for the ingest kernels (transform, tiles, samples).
+ * Results do not depend on them; speed does.  sbki_set_tuning drops the recorded
  * batched updates (they are recorded again with the new shapes). */
 typedef struct sbki_tuning {
   int32_t accumulate_ctas_per_sm;

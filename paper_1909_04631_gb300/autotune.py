@@ -1,7 +1,7 @@
 """Autotuner of the update's launch shapes.
 
 The kernels of the update run on persistent grids whose shapes (CTAs per SM
-of the accumulation, training points per warp chunk, CTAs per SM of the
+of the accumulation, pairs of training points per warp chunk, CTAs per SM of the
 touched-block pass and of the ingest kernels) change speed, not results; so
 does the form of the accumulation (point-major or block-major: the same keys
 and pair counts, alpha up to the order of FP32 sums).  `autotune` times

@@ -57,7 +57,7 @@ struct PtArgs {
   int tpad;              // entries per list (multiple of 32)
   int R;                 // offsets per axis span [-R, R]
   uint32_t recip_na;     // small_recip(2R + 1)
-  int chunk;             // consecutive training points per warp (fast form)
+  int chunk;             // consecutive training points per warp at most (fast form)
   int32_t sink;          // spare pool block that absent neighbour blocks point at
   const uint16_t* ftab;  // fast form: [tables][kFastLists][list_pad] entries, then a list of padding entries
   const int32_t* flen;   // [tables][kFastLists] entries of each list
@@ -585,8 +585,9 @@ cudaError_t upload_lists(const std::vector<T>& flat, const std::vector<int32_t>&
 
 }  // namespace
 
-// Candidate lists (host, once per map): kParts^3 lists in the general form and,
-// when 2R + 1 <= 7, kFastParts^3 lists in the fast form's entry format.
+// Candidate lists (host, once per map): kParts^3 lists of voxels in the general
+// form and, for supports of at most 7 offsets per axis, kFastLists lists of pairs
+// of voxels per distinct class support in the fast form.
 cudaError_t build_candidate_tables(MapState& m) {
   const double lr = m.prm.length_scale / m.prm.res;
   std::vector<std::vector<int32_t>> lists;
@@ -745,7 +746,7 @@ cudaError_t launch_accumulate_points(MapState& m) {
   a.tpad = m.ctab_pad;
   a.R = m.ctab_R;
   a.recip_na = ((1u << 20) + (uint32_t)(2 * m.ctab_R + 1) - 1u) / (uint32_t)(2 * m.ctab_R + 1);
-  // whole groups of kGroup points; the kernel takes fewer where there are few points
+  // the tuning counts pairs of points; whole groups of kGroup points; the kernel takes fewer where there are few points
   a.chunk = (2 * std::max(1, std::min(64, m.tune.accumulate_chunk)) + kGroup - 1) / kGroup * kGroup;
   // soft labels: a point with a weight row costs up to K+1 times the reductions, so smaller
   // chunks balance the work queue better (16 against 60 points: 413 against 477 us per street scan)

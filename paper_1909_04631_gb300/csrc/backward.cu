@@ -272,8 +272,9 @@ __global__ void __launch_bounds__(kThreads, 3) backward_kernel(BwdArgs a) {
 //
 // Bound by instruction issue, as the accumulation's sweep is.  2.0M points,
 // 223M pairs: one voxel per lane with FP64 sums per point took 1378 us, this
-// form takes 905.  The largest part of the difference are the FP64 sums: two
-// fused multiply-adds per point and lane hold the SM's FP64 units for ~900 us.
+// form 905 with the pairs kept to the end and about 14 more as it is.  The largest
+// part of the difference are the FP64 sums: two fused multiply-adds per point and
+// lane hold the SM's FP64 units for ~900 us.
 constexpr int kBwdChunk = 16;  // consecutive training points per warp
 constexpr int kBwdFold = 4;    // chunks whose sums are held in FP32 pairs
 

@@ -319,7 +319,7 @@ __device__ __forceinline__ uint32_t touched_digits(const float4& p, const int v0
     if (touches64(p, v0, d, g, sup.l2_64)) in |= 1u << d;
   }
   // extended-block association: the own block and its face neighbours
-  return g.assoc ? in & (1u << 4 | 1u << 10 | 1u << 12 | 1u << 13 | 1u << 14 | 1u << 16 | 1u << 22) : in;
+  return g.assoc ? in & kFaceDigits : in;
 }
 
 // For the fast accumulation form: every point's own block (always touched: the

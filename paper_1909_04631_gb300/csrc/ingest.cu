@@ -19,8 +19,6 @@
 namespace sbki {
 namespace {
 
-
-
 // sort key: [scan | rel tile x | rel tile y | rel tile z | local cell (z,y,x) | label]
 __device__ __forceinline__ unsigned long long make_key(float x, float y, float z, int label, const Geom& g,
                                                        const KeyFrame& kf, const int32_t org[3], int scan,

@@ -377,7 +377,9 @@ cudaError_t launch_downsample_n(MapState& m, const KeyFrame& kf, int64_t nitems)
 // scratch (tile_frame_fits), the items leave room for the flagged points
 // (item_cap), and the occupied tiles not exceed TileGate::limit.
 constexpr uint32_t kTilesDeclined = 1u << 30;  // an item outside the frame, or in a cell beyond 2^22
-constexpr int64_t kTileFrameMax = 1 << 22;  // directory entries per scan at most
+// directory entries per scan at most: 10 us of them (TileGate), a max_range of 62 m
+// at 0.1 m cells.  Larger frames are fitted to the hits after the counters' read-back
+constexpr int64_t kTileFrameMax = 1 << 22;
 int64_t tile_capacity(int64_t sample_capacity);
 // Whether an update whose tiles were marked is the tile form's, on the host and
 // on the device (one decision: integers only).

@@ -29,9 +29,11 @@
 // beams' items is three reductions and two dependent lookups into tables that
 // stay in L2.  Ingest of a 64 x 2048 street scan (3.0M items, 690k points)
 // 348 -> 239 us, of a 640 x 480 depth frame (9.3M items, 300k points) 822 -> 354,
-// of a 9k-ray scan 153 -> 134, of 16 street scans in a batch 2600 -> 1490.
+// of a 9k-ray scan 153 -> 122, of 16 street scans in a batch 2600 -> 1490.
 // What bounds it: the reductions (40 of the 85 us of `add` on the street scan)
-// and the issue of forming each item three times.
+// and the issue of forming each item three times; for sparse scans the cells of
+// their tiles, for few beams the walk along the longest.  There, and for beams in
+// no order, the sorted form is the faster one: TileGate draws the line.
 #include <algorithm>
 #include <cmath>
 
