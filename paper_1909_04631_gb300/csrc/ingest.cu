@@ -133,7 +133,9 @@ __device__ __forceinline__ void finish_counts(unsigned long long total, int64_t 
 }
 
 // Steps a1 (and the free-sample counts of a2) for every point of every scan
-// of the update; points are numbered globally, scan after scan.
+// of the update; points are numbered globally, scan after scan.  kTiles: and what
+// TileGate asks of the beams (the longest, those beside the next).
+template <bool kTiles>
 __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __restrict__ desc, int ns, Geom g,
                                                                float4* __restrict__ world,
                                                                unsigned long long* __restrict__ cnt, int64_t items_cap,
@@ -159,11 +161,13 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
     int tile[3] = {INT_MIN / 2, 0, 0};  // of a kept hit
     if (i < total) c = transform_count_one(desc[scan_of(s_off, ns, i)], i, s_off, g, world, cnt, dc, tile, tlo, thi);
     sum += c;
-    longest = max(longest, (uint32_t)(c & kFreeMask));
-    int apart = 0;  // tiles to the next point's hit
+    if (kTiles) {
+      longest = max(longest, (uint32_t)(c & kFreeMask));
+      int apart = 0;  // tiles to the next point's hit
 #pragma unroll
-    for (int a = 0; a < 3; ++a) apart = max(apart, abs(tile[a] - __shfl_down_sync(0xffffffffu, tile[a], 1)));
-    near += apart <= 1 && c != 0ull && (threadIdx.x & 31) != 31 ? 1u : 0u;
+      for (int a = 0; a < 3; ++a) apart = max(apart, abs(tile[a] - __shfl_down_sync(0xffffffffu, tile[a], 1)));
+      near += apart <= 1 && c != 0ull && (threadIdx.x & 31) != 31 ? 1u : 0u;
+    }
   }
   // tile bounding box of the kept hits: warp, then CTA, then one global atomic per CTA and bound
 #pragma unroll
@@ -176,19 +180,23 @@ __global__ void __launch_bounds__(256) transform_count_kernel(const ScanDesc* __
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-  longest = __reduce_max_sync(0xffffffffu, longest);
-  near = __reduce_add_sync(0xffffffffu, near);
+  if (kTiles) {
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    near = __reduce_add_sync(0xffffffffu, near);
+  }
   if ((threadIdx.x & 31) == 0 && sum) {
     atomicAdd(&s_total, sum);
-    atomicMax(&s_longest, longest);
-    atomicAdd(&s_near, near);
+    if (kTiles) {
+      atomicMax(&s_longest, longest);
+      atomicAdd(&s_near, near);
+    }
   }
   __syncthreads();
   if (threadIdx.x < 3 && s_box[threadIdx.x] <= s_box[3 + threadIdx.x]) {
     atomicMin(&dc->tbox[threadIdx.x], s_box[threadIdx.x]);
     atomicMax(&dc->tbox[3 + threadIdx.x], s_box[3 + threadIdx.x]);
   }
-  if (threadIdx.x == 32 && s_total) {  // read by later launches
+  if (kTiles && threadIdx.x == 32 && s_total) {  // read by later launches
     atomicMax(&dc->longest, s_longest);
     atomicAdd(&dc->n_near, s_near);
   }
@@ -836,9 +844,10 @@ inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + thread
 
 // Steps a1-a2 count for the ns scans described in m.s.desc; total_n bounds the
 // point count, which the kernels read on the device (dc->n_points, desc[ns].off).
-cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n) {
+cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n, bool tiles) {
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(grid_for(total_n, 256), (int64_t)m.sm_count * m.tune.ingest_ctas_per_sm));
-  transform_count_kernel<<<blocks, 256, 0, m.stream>>>(m.s.desc, ns, m.g, m.s.world, m.s.cnt, m.s.s_cap, m.dc);
+  auto* kernel = tiles ? transform_count_kernel<true> : transform_count_kernel<false>;
+  kernel<<<blocks, 256, 0, m.stream>>>(m.s.desc, ns, m.g, m.s.world, m.s.cnt, m.s.s_cap, m.dc);
   m.launches += 1;
   return cudaGetLastError();
 }

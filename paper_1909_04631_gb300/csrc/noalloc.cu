@@ -200,7 +200,7 @@ sbki_status run(const sbki_params* params, const float* points, const int32_t* l
   }
   hd[1].off = n;
   CKN(cudaMemcpyAsync(s.desc, hd, sizeof(hd), cudaMemcpyHostToDevice, m.stream));
-  CKN(launch_transform_count(m, 1, n));
+  CKN(launch_transform_count(m, 1, n, false));
   CKN(launch_offsets(m, n));
   DevCounters h;
   CKN(cudaMemcpyAsync(&h, m.dc, sizeof(h), cudaMemcpyDeviceToHost, m.stream));

@@ -128,6 +128,7 @@ __global__ void begin_kernel(DevCounters* dc, uint32_t epoch, uint32_t n_points)
   dc->n_scan = 0;
   dc->n_total = 0;
   dc->n_ttiles = 0;
+  dc->tiles_taken = 0;
   dc->longest = 0;
   dc->n_near = 0;
   dc->n_wide = 0;
@@ -161,6 +162,7 @@ __global__ void batch_begin_kernel(DevCounters* dc, const ScanDesc* desc, int ns
   dc->n_scan = 0;
   dc->n_total = 0;
   dc->n_ttiles = 0;
+  dc->tiles_taken = 0;
   dc->longest = 0;
   dc->n_near = 0;
   dc->n_wide = 0;
@@ -480,7 +482,7 @@ sbki_status run_ingest(MapState& m, const float* points, const int32_t* labels, 
   m.hdesc[1] = ScanDesc{};
   m.hdesc[1].off = n;
   CK(&m, cudaMemcpyAsync(m.s.desc, m.hdesc, 2 * sizeof(ScanDesc), cudaMemcpyHostToDevice, m.stream));
-  CK(&m, launch_transform_count(m, 1, n));
+  CK(&m, launch_transform_count(m, 1, n, !probs));
   // The tile form (soft labels need the sorted items).  Where the frame of
   // max_range fits a directory, the tiles are marked before the counters come
   // back, so the read-back also tells how many are occupied (or that items lie
@@ -962,7 +964,7 @@ sbki_status sbki_insert_batch(sbki_map* map, const sbki_scan* scans, int32_t cou
     }
     batch_begin_kernel<<<1, 1, 0, m.stream>>>(m.dc, m.s.desc, count);
     m.launches += 1;
-    cudaError_t ce = launch_transform_count(m, count, m.s.n_cap);
+    cudaError_t ce = launch_transform_count(m, count, m.s.n_cap, true);
     // the tile form where the scans' frames fit, then the sorted form for what it leaves (as a rule nothing)
     if (ce == cudaSuccess && tile_frame_fits(m, count, kf)) {
       ce = launch_tile_mark(m, count, m.s.n_cap, kf, false);

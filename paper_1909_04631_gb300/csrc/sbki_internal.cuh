@@ -57,6 +57,7 @@ struct DevCounters {
   uint32_t transform_done;            // CTAs of the transform finished (the last one adds up the counts)
   unsigned long long n_total;         // hits << 40 | free samples of this scan
   uint32_t n_ttiles;                  // tile form: occupied tiles (kTilesDeclined and more: not this form)
+  uint32_t tiles_taken;               // 1: the tile form has this update
   uint32_t n_low;                     // tile form: fractions noted
   uint32_t n_wide;                    // tile form: training points left to the gathered exact mean
   uint32_t n_gather;                  // tile form: their members
@@ -368,7 +369,8 @@ cudaError_t radix_wait_selftest(unsigned long long* keys, uint32_t* vals, unsign
 
 // ingest.cu
 // ingest of the ns scans described in m.s.desc (ns + 1 entries, the last holding the total)
-cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n);
+// (tiles: the tile form may follow)
+cudaError_t launch_transform_count(MapState& m, int ns, int64_t total_n, bool tiles);
 // sorted form: the points' counts to offsets (the tile form reads the counts), then the items
 cudaError_t launch_offsets(MapState& m, int64_t total_n);
 cudaError_t launch_emit(MapState& m, int ns, int64_t total_n, const KeyFrame& kf, uint32_t* hit_src = nullptr);
@@ -389,18 +391,19 @@ int64_t tile_capacity(int64_t sample_capacity);
 // tile form gains, in tiles of 2.55 us per 1000 (4 KB of cells each, cleared,
 // counted and given offsets): 0 to 39 us by the items (few items sort quickly) and
 // 45 us per million items of beams that lie beside the next ones (others: nothing;
-// n_near tells); it loses 0.25 us per sample of the longest beam above 50 (three
-// passes walk along it) and 2.4 us per million directory entries.  From 63 scans
-// of 34 to 8.3M items, up to 199k tiles and 200 samples a beam, and 8 batches, both
-// forms measured, in us sorted / tiles.  Ingest: 165 items of one 50 m beam 92 /
-// 119; 12k of 500 such beams 134 / 138; 8400 of 500 beams of 15 m 133 / 100; 79k
-// items in 2600 tiles 146 / 112; 3.1M in 6300 351 / 221; 916k in 44k, beams in
-// random order, 205 / 314; 215k in 55k 170 / 321.  Batches of 16: 1.1M items in 50k
-// tiles 401 / 534, 11M in 88k 1375 / 1111.  An update declined after marking pays
-// 20 to 50 us for it, so the line lies 8000 tiles above `even`, where the forms are
-// equal (at `even`, shuffled street scans took 263 and 425 us for 249 and 379);
-// where that is no tile at all marking does not start (0), which leaves two idle
-// launches, about 7 us.
+// n_near tells); it loses 0.2 us per sample of the longest beam above 50 (three
+// passes walk along it) and 1.2 to 2.4 us per million directory entries.  From 63
+// scans of 34 to 8.3M items, up to 199k tiles and 200 samples a beam, and 23
+// batches, both forms measured, in us sorted / tiles.  Ingest: 165 items of one
+// 50 m beam 93 / 119; 12k of 500 such beams 135 / 137; 10k of 500 beams of 30 m
+// 134 / 111; 79k items in 2600 tiles 146 / 112; 3.1M in 6300 351 / 220; 916k in
+// 44k, beams in random order, 204 / 313; 216k in 55k 169 / 320.  Whole batches: 3
+// scans, 505k items in 14k tiles 238 / 251; 13 scans, 1.8M in 59k 467 / 568, 4.6M
+// in 66k 715 / 737; 16 scans, 11M in 88k 1362 / 1104.
+// An update declined after marking pays 20 to 75 us for it (more with a larger
+// directory), so it is declined only 8000 tiles above the line where the forms are
+// equal, and the directory's own share counts only for whether marking starts at
+// all (where it does not, the limit is 0 and two idle launches stay, about 7 us).
 struct TileGate {
   uint32_t tile_cap, item_cap;
   uint32_t entries;  // of the directory
@@ -409,8 +412,9 @@ struct TileGate {
     const uint32_t beside = c.n_valid ? 32u * c.n_near / c.n_valid : 0u;  // of 32
     const uint32_t gain = 15360u * few / (few + 2304u) + c.n_items / 64u * beside / 32u;
     const uint32_t longest = c.longest < 50u ? 0u : (c.longest < 200000u ? c.longest - 50u : 200000u);
-    const int32_t even = (int32_t)gain - (int32_t)(98u * longest + entries / 1024u);
-    return even <= 0 ? 0u : ((uint32_t)even + 8192u < tile_cap ? (uint32_t)even + 8192u : tile_cap);
+    if (gain <= 80u * longest + entries / 1024u) return 0u;
+    const uint32_t most = gain - 80u * longest + 8192u;
+    return most < tile_cap ? most : tile_cap;
   }
   __host__ __device__ bool takes(const DevCounters& c) const {
     return c.err == 0 && c.n_ttiles <= limit(c) && c.n_items <= item_cap;

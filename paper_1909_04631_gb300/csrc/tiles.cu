@@ -250,9 +250,9 @@ __device__ __forceinline__ void each_item(const TileArgs& a, Op& op) {
   }
 }
 
-// whether the tile form takes this update (decided on the device; n_sort holds the answer
-// for the sorted form)
-__device__ __forceinline__ bool tiles_on(const TileArgs& a) { return a.gate.takes(*a.dc); }
+// whether the tile form takes this update: decided on the device when its tiles are marked
+// (tile_rank_kernel; n_sort holds the answer for the sorted form)
+__device__ __forceinline__ bool tiles_on(const TileArgs& a) { return a.dc->tiles_taken != 0u; }
 __device__ __forceinline__ bool packed(const TileArgs& a) { return a.dc->max_points < a.pack_limit; }
 
 // ---------------------------------------------------------------- mark, rank
@@ -298,10 +298,14 @@ struct MarkOp {
     }
   }
 };
-// The directory and its counts to zero, unless marking will not start.
+// The directory and its counts to zero, unless marking will not start.  Up to
+// kClearAlways words a plain memset takes no longer than this launch.
+constexpr int64_t kClearAlways = 1 << 18;
 __global__ void __launch_bounds__(256) tile_clear_kernel(TileArgs a, uint32_t words) {
-  if (a.dc->err || a.dc->n_ttiles > a.gate.limit(*a.dc)) return;  // neither changes in this launch
-  if (a.gate.limit(*a.dc) == 0u) return;
+  __shared__ uint32_t s_limit;  // nothing of it changes in this launch
+  if (threadIdx.x == 0) s_limit = a.dc->err || a.dc->n_ttiles ? 0u : a.gate.limit(*a.dc);
+  __syncthreads();
+  if (s_limit == 0u) return;
   uint4* const d = reinterpret_cast<uint4*>(a.b.dir);
   const uint32_t i0 = blockIdx.x * 256 + threadIdx.x;
   for (uint32_t i = i0; i < words / 4; i += gridDim.x * 256) d[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -311,17 +315,15 @@ __global__ void __launch_bounds__(256) tile_clear_kernel(TileArgs a, uint32_t wo
 __global__ void __launch_bounds__(256, 6) tile_mark_kernel(TileArgs a) {
   // other CTAs of this launch may set the error, decline or pass the limit, so one read decides for the whole CTA:
   // warps that went on without the others would miss each_item's scan offsets
-  __shared__ int s_off;
-  const uint32_t limit = a.gate.limit(*a.dc);
+  __shared__ uint32_t s_limit;  // 0: nothing to do
   if (threadIdx.x == 0) {
-    s_off = *(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles > limit;
-    if (limit == 0u) {  // not even one tile
-      atomicMax(&a.dc->n_ttiles, kTilesDeclined);
-      s_off = 1;
-    }
+    s_limit = a.gate.limit(*a.dc);
+    if (s_limit == 0u) atomicMax(&a.dc->n_ttiles, kTilesDeclined);  // not even one tile
+    if (*(volatile const int*)&a.dc->err != 0 || *(volatile const uint32_t*)&a.dc->n_ttiles > s_limit) s_limit = 0u;
   }
   __syncthreads();
-  if (s_off) return;
+  const uint32_t limit = s_limit;
+  if (limit == 0u) return;
   MarkOp op{a, limit};
   each_item(a, op);
   const uint32_t w = __reduce_add_sync(0xffffffffu, op.fresh);
@@ -352,15 +354,19 @@ __device__ __forceinline__ int tile_of_entry(const TileArgs& a, uint32_t e, int 
 // its tiles are cleared.  n_sort: the items left to the sorted form.
 __global__ void __launch_bounds__(256) tile_rank_kernel(TileArgs a) {
   __shared__ uint32_t s_w[8];
-  if (blockIdx.x == 0 && threadIdx.x == 0 && tiles_on(a)) a.dc->n_sort = a.dc->n_scan = 0u;
-  if (!tiles_on(a)) return;
+  if (!a.gate.takes(*a.dc)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.dc->tiles_taken = 1u;
+    a.dc->n_sort = a.dc->n_scan = 0u;
+  }
   const uint32_t nch = (a.b.entries + kChunk - 1) / kChunk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t whole = 0u, next = threadIdx.x;  // this thread's share of the second-level counts, read once as c grows
   for (uint32_t c = blockIdx.x; c < nch; c += gridDim.x) {
     if (a.b.chunks[c] == 0u) continue;  // uniform over the CTA
     __syncthreads();
-    uint32_t before = 0;
-    for (uint32_t k = threadIdx.x; k < c / kSuper; k += 256) before += a.b.supers[k * kSuperStep];
+    for (; next < c / kSuper; next += 256) whole += a.b.supers[next * kSuperStep];
+    uint32_t before = whole;
     for (uint32_t k = c / kSuper * kSuper + threadIdx.x; k < c; k += 256) before += a.b.chunks[k];
     before = __reduce_add_sync(0xffffffffu, before);
     if (lane == 0) s_w[warp] = before;
@@ -868,10 +874,16 @@ cudaError_t launch_tile_mark(MapState& m, int ns, int64_t total_n, const KeyFram
   const uint32_t entries = (uint32_t)((int64_t)kf.ext[0] * kf.ext[1] * kf.ext[2] * ns);
   const TileArgs a = tile_args(m, ns, entries, kf, alone);
   const int64_t words = directory_words(entries, a.b.tile_cap);
-  const unsigned blocks = (unsigned)std::min<int64_t>((words / 4 + 255) / 256 + 1, (int64_t)m.sm_count * 8);
-  tile_clear_kernel<<<blocks, 256, 0, m.stream>>>(a, (uint32_t)words);
+  if (words <= kClearAlways) {
+    const cudaError_t e = cudaMemsetAsync(a.b.dir, 0, sizeof(uint32_t) * (size_t)words, m.stream);
+    if (e != cudaSuccess) return e;
+  } else {
+    const unsigned blocks = (unsigned)std::min<int64_t>((words / 4 + 255) / 256 + 1, (int64_t)m.sm_count * 8);
+    tile_clear_kernel<<<blocks, 256, 0, m.stream>>>(a, (uint32_t)words);
+    m.launches += 1;
+  }
   tile_mark_kernel<<<item_blocks(m, total_n), 256, 0, m.stream>>>(a);
-  m.launches += 2;
+  m.launches += 1;
   return cudaGetLastError();
 }
 
