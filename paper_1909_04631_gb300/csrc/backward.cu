@@ -272,9 +272,8 @@ __global__ void __launch_bounds__(kThreads, 3) backward_kernel(BwdArgs a) {
 //
 // Bound by instruction issue, as the accumulation's sweep is.  2.0M points,
 // 223M pairs: one voxel per lane with FP64 sums per point took 1378 us, this
-// form 905 with the pairs kept to the end and about 14 more as it is.  The largest
-// part of the difference are the FP64 sums: two fused multiply-adds per point and
-// lane hold the SM's FP64 units for ~900 us.
+// form takes 905.  The largest part of the difference are the FP64 sums: two
+// fused multiply-adds per point and lane hold the SM's FP64 units for ~900 us.
 constexpr int kBwdChunk = 16;  // consecutive training points per warp
 constexpr int kBwdFold = 4;    // chunks whose sums are held in FP32 pairs
 
@@ -355,19 +354,17 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
       const int gn = (int)min(c1 - g0, (int64_t)kGroup);  // warp-uniform
       // rows of every point of the group, four lanes per point
       int pt = 0, lw = 0, b0 = 0;
-      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (gl < gn) p = a.xyzl[g0 + gl];
-      float x = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
-      // A coordinate that is not finite or past floor_small's range reaches no voxel of a map.  Every candidate is
-      // multiplied out below, masked or not, so such a point's rows must not hold it (0 * inf is NaN): they are formed
-      // at 0 and the point takes no list.
-      const bool inside = fabsf(__fmul_rn(x, g.inv_res)) < 4194304.0f;
-      const uint32_t insides = __ballot_sync(0xffffffffu, inside);
-      if (!inside) x = 0.f;
       if (gl < gn) {
-        const AxisFrame f = axis_frame(x, g);
+        const float4 p = a.xyzl[g0 + gl];
+        const float x = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
+        // A coordinate that is not finite or past floor_small's range reaches no voxel of a map.  Every candidate is
+        // multiplied out below, masked or not, so such a point's rows must not hold it (0 * inf is NaN): they are
+        // formed at 0 and the point has no list.
+        const bool inside = fabsf(__fmul_rn(x, g.inv_res)) < 4194304.0f;
+        const AxisFrame f = axis_frame(inside ? x : 0.f, g);
         lw = label_of(p.w);
         pt = form_rows<false>(W.slot[gl], gl, role, f, (uint32_t)((lw & ((1 << kLabelBits) - 1)) * g.B3), R, g);
+        if (!inside) pt = kFastLists;
         b0 = f.v0 >> g.B_shift;
       }
       const int pty = __shfl_sync(0xffffffffu, pt, lane | 2), ptz = __shfl_sync(0xffffffffu, pt, lane | 3);
@@ -376,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
         const int list = pt + kFastParts * (pty + kFastParts / 2 * ptz);
         const int label = lw & ((1 << kLabelBits) - 1), map = lw >> kLabelBits;
         // others have no G
-        const bool known = label < g.K1 && map < kMaxMaps && ((insides >> lane) & 15u) == 15u;
+        const bool known = label < g.K1 && map < kMaxMaps && list < kFastLists;
         const unsigned long long key = known ? pack_block(b0, by, bz, map) : kEmpty;
         uint32_t* sc = reinterpret_cast<uint32_t*>(W.slot[gl] + kScalars);
         sc[0] = known ? (uint32_t)(list * a.list_pad) : a.pad_list;
