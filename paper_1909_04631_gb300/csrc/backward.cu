@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(kThreads, 3) backward_kernel(BwdArgs a) {
 // FP32.  FP64 runs at 1/64 of the FP32 rate on this chip, so a lane sums the
 // points of a few chunks as unevaluated FP32 pairs (error-free sums and
 // products, 2^-44 relative over its 32 points) and then adds them to an FP64
-// sum: neither the range nor the error depends on the length of the set (after
-// every chunk it costs 1 % more).
+// sum of its own in shared memory (in registers: 921 us instead of 905 below):
+// neither the range nor the error depends on the length of the set.
 //
 // Bound by instruction issue, as the accumulation's sweep is.  2.0M points,
 // 223M pairs: one voxel per lane with FP64 sums per point took 1378 us, this
@@ -315,6 +315,7 @@ template <bool kClass>
 __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) {
   __shared__ BwdWarp s_w[kWarps];
   __shared__ double s_cls[kClass ? kWarps : 1][32];  // per warp: sum G f by class
+  __shared__ double s_sum[kWarps][2][32];            // per lane: sum s G f, sum s G u^4 D d
   extern __shared__ __align__(16) uint16_t s_lists[];
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
   PairSum acc_f, acc_l;              // sum s G f, sum s G u^4 D d, by column
   acc_f.clear();
   acc_l.clear();
-  double af = 0.0, al = 0.0;         // their sums over this lane's chunks
+  s_sum[wid][0][lane] = s_sum[wid][1][lane] = 0.0;
   int chunks = 0;
   const int64_t gw = (int64_t)blockIdx.x * kWarps + wid, nw = (int64_t)gridDim.x * kWarps;
   for (int64_t c = gw; c * kBwdChunk < a.p; c += nw) {
@@ -480,12 +481,11 @@ __global__ void __launch_bounds__(kThreads, 3) backward_pairs_kernel(BwdArgs a) 
       __syncwarp();  // the slots are rewritten by the next group
     }
     if (++chunks % kBwdFold == 0) {  // warp-uniform
-      af += acc_f.take();
-      al += acc_l.take();
+      s_sum[wid][0][lane] += acc_f.take();
+      s_sum[wid][1][lane] += acc_l.take();
     }
   }
-  af += acc_f.take();
-  al += acc_l.take();
+  double af = s_sum[wid][0][lane] + acc_f.take(), al = s_sum[wid][1][lane] + acc_l.take();
   for (int o = 16; o > 0; o >>= 1) {
     af += __shfl_down_sync(0xffffffffu, af, o);
     al += __shfl_down_sync(0xffffffffu, al, o);
